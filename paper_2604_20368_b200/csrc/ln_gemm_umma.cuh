@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(256, 3) k_nn_umma(const float* __restrict__ E,
   };
   fetch(0);
   for (int kb = 0; kb < nkb; ++kb) {
-    if (tid == 0) {                              // the Y block arrives while the E block is converted
+    if (umma::leader(tid)) {                     // the Y block arrives while the E block is converted
       umma::mbar_expect_tx(&mbar_y, 2 * GU_KB * D * 2);
       umma::bulk_load(sY, Yimg + (long long)kb * (2 * GU_KB * D), 2 * GU_KB * D * 2, &mbar_y);
     }
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(256, 3) k_nn_umma(const float* __restrict__ E,
     umma::fence_smem_to_mma();
     __syncthreads();
     if (kb + 1 < nkb) fetch(kb + 1);             // in flight while the MMAs of this block run
-    if (tid == 0) {
+    if (umma::leader(tid)) {
       ok &= umma::mbar_wait(&mbar_y, ph_y & 1);
       umma::fence_after_sync();
 #pragma unroll 1
@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(256, 2) k_ntg_umma(const bf16* __restrict__ U,
   umma::fence_after_sync();
   const uint32_t tacc = tmem_base;
   constexpr uint32_t YB = 2 * GU_KB * D * 2;     // bytes of one block (hi + lo)
-  if (tid == 0)                                  // the first two blocks are on their way while the U tile is copied
+  if (umma::leader(tid))                         // the first two blocks are on their way while the U tile is copied
     for (int nb = 0; nb < 2 && nb < nkb; ++nb) {
       umma::mbar_expect_tx(&mbar_y[nb], YB);
       umma::bulk_load(sY + nb * (2 * GU_KB * D), Yimg + (long long)nb * (2 * GU_KB * D), YB, &mbar_y[nb]);
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(256, 2) k_ntg_umma(const bf16* __restrict__ U,
   };
   fetch_e(0);
   bool ok = true;
-  if (tid == 0) {
+  if (umma::leader(tid)) {
     const uint32_t idesc = umma::instr_desc(GU_KB, false, false);
     uint32_t ph_y[2] = {0, 0}, ph_f[2] = {0, 0};
     for (int nb = 0; nb < nkb; ++nb) {

@@ -57,15 +57,15 @@ __device__ __forceinline__ void umma_gemm(uint32_t tmem_d, const bf16* A, bool a
   }
 }
 
-// issue (thread 0) + wait (everyone); returns false on a timed-out wait
+// issue (one thread) + wait (everyone); returns false on a timed-out wait
 // `phase` is each thread's own copy of the mbarrier phase (identical in all threads)
-// drain_stores: thread 0 first lets its bulk stores finish reading shared memory, so that when the barrier
+// drain_stores: the issuing thread first lets its bulk stores finish reading shared memory, so that when the barrier
 // completes the buffers those stores read may be overwritten by everybody
 template <int UM>
 __device__ __forceinline__ bool umma_run(UmmaCtl& ctl, uint32_t& phase, uint32_t tmem_d, const bf16* A, bool a_k, const bf16* Bm,
                                          bool b_k, bool accumulate, const bf16* A2 = nullptr, bool a2_k = true,
                                          const bf16* B2 = nullptr, bool b2_k = true, bool drain_stores = false) {
-  if (threadIdx.x == 0) {
+  if (umma::leader(threadIdx.x)) {
     umma::fence_after_sync();
     umma_gemm<UM>(tmem_d, A, a_k, Bm, b_k, accumulate);
     if (A2) umma_gemm<UM>(tmem_d, A2, a2_k, B2, b2_k, true);
@@ -204,7 +204,7 @@ __device__ bool ns_forward_umma(int m, int T, float eps, float alpha_in, const f
   }
   bool ok = true;
   umma_step_done(ctl, true);
-  if (tid == 0 && T > 0) umma::bulk_store(Xh, sX, MATB);                                   // image of X_0
+  if (umma::leader(tid) && T > 0) umma::bulk_store(Xh, sX, MATB);                                   // image of X_0
   for (int k = 0; k < T; ++k) {
     // the store of Q_{k-1} has read sP before the barrier of this product completes
     ok &= umma_run<UM>(ctl, phase, ctl.tmem_base, sW, true, sX, false, false, nullptr, true, nullptr, true, true);   // D = W X_k
@@ -218,7 +218,7 @@ __device__ bool ns_forward_umma(int m, int T, float eps, float alpha_in, const f
       }
     }
     umma_step_done(ctl, ok);
-    if (tid == 0 && Ph) umma::bulk_store(Ph + k * hs, sP, MATB);
+    if (umma::leader(tid) && Ph) umma::bulk_store(Ph + k * hs, sP, MATB);
     // the store of X_k has read sX before the barrier of this product completes
     ok &= umma_run<UM>(ctl, phase, ctl.tmem_base, sX, true, sP, false, false, nullptr, true, nullptr, true, true);   // D = X_k Q_k
     {
@@ -234,9 +234,9 @@ __device__ bool ns_forward_umma(int m, int T, float eps, float alpha_in, const f
       }
     }
     umma_step_done(ctl, ok);
-    if (tid == 0 && k + 1 < T) umma::bulk_store(Xh + (k + 1) * hs, sX, MATB);
+    if (umma::leader(tid) && k + 1 < T) umma::bulk_store(Xh + (k + 1) * hs, sX, MATB);
   }
-  if (tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");      // every image has reached global memory
+  if (umma::leader(tid)) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");      // every image has reached global memory
   ok &= (ctl.timeout == 0);
   umma_end(ctl, UM);
   return ok;
@@ -270,7 +270,7 @@ __device__ bool ns_backward_umma(int m, int T, float eps, const float* W, const 
   uint32_t phase = 0, ph_ld = 0;
   const uint32_t t_acc = ctl.tmem_base, t_dw = ctl.tmem_base + UM;
   auto load_image = [&](const float* src) {     // one thread starts the copy into sA
-    if (tid == 0) {
+    if (umma::leader(tid)) {
       umma::mbar_expect_tx(&ctl.mbar_ld, MATB);
       umma::bulk_load(sA, src, MATB, &ctl.mbar_ld);
     }
@@ -281,7 +281,7 @@ __device__ bool ns_backward_umma(int m, int T, float eps, const float* W, const 
     return got;
   };
   auto load_pair = [&](int k) {                 // A = X_k and Q_k, counted on one phase of the barrier
-    if (tid == 0) {
+    if (umma::leader(tid)) {
       umma::mbar_expect_tx(&ctl.mbar_ld, 2 * MATB);
       umma::bulk_load(sA, Xh + (long long)k * hs, MATB, &ctl.mbar_ld);
       umma::bulk_load(sQ, Ph + (long long)k * hs, MATB, &ctl.mbar_ld);
@@ -304,7 +304,7 @@ __device__ bool ns_backward_umma(int m, int T, float eps, const float* W, const 
     }
     umma_step_done(ctl, ok);
     if constexpr (QBUF) {
-      if (tid == 0) {
+      if (umma::leader(tid)) {
         umma::fence_after_sync();
         umma_gemm<UM>(t_dw, sH, true, sA, true, k != T - 1);                                  // dW accumulator += H A^T
         umma_gemm<UM>(t_acc, sG, true, sQ, true, false);                                      // G Q^T

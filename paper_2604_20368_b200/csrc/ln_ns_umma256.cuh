@@ -44,8 +44,8 @@ struct U2Ctx {
   UmmaCtl* ctl; unsigned long long* mbar_x; unsigned long long* mbar_y;   // S x has completed; S y (and S x) have completed
   unsigned long long* mbar_ldy;                 // arrival of the y block (S and x are counted on ctl->mbar_ld)
   bf16* buf[3];
-  uint32_t phase, ph_ld, ph_ldy, ph_x, ph_y;    // ph_ld / ph_ldy / ph_x / ph_y are used by thread 0 only
-  bool pre;                                     // thread 0: the first S block of the next product is on its way into buffer 2
+  uint32_t phase, ph_ld, ph_ldy, ph_x, ph_y;    // ph_ld / ph_ldy / ph_x / ph_y are used by the issuing thread only
+  bool pre;                                     // issuing thread: the first S block of the next product is on its way into buffer 2
   bool ok;
 };
 
@@ -61,7 +61,7 @@ __device__ __forceinline__ void u2_fence_async() { asm volatile("fence.proxy.asy
 template <int NG>
 __device__ __forceinline__ void u2_run(U2Ctx& c, const U2Group (&g)[NG], const bf16* next_S = nullptr) {
   constexpr uint32_t MATB = (uint32_t)kUmmaMatBytes;
-  if (threadIdx.x == 0) {
+  if (umma::leader(threadIdx.x)) {
     int is = 0, ix = 1, iy = 2;                                       // buffers of S, x, y of the current group
     u2_fence_async();
     if (c.pre) {                                                       // S is on its way (its bytes and x's were announced then)
@@ -110,7 +110,7 @@ __device__ __forceinline__ void u2_run(U2Ctx& c, const U2Group (&g)[NG], const b
   c.ok &= umma::mbar_wait(&c.ctl->mbar, c.phase & 1);
   c.phase ^= 1u;
   umma::fence_after_sync();
-  if (threadIdx.x == 0) {
+  if (umma::leader(threadIdx.x)) {
     c.pre = next_S != nullptr;
     if (next_S) {                                                      // every buffer has been read; the epilogue uses 0 and 1
       umma::mbar_expect_tx(&c.ctl->mbar_ld, 2 * MATB);
@@ -127,7 +127,7 @@ __device__ __forceinline__ void u2_store_block(U2Ctx& c, const float (&v)[64], i
   umma::fence_smem_to_mma();
   umma::fence_before_sync();
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (umma::leader(threadIdx.x)) {
     umma::bulk_store(dst, c.buf[b], (uint32_t)kUmmaMatBytes);
     if (last) {
       asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
@@ -230,7 +230,7 @@ __device__ bool ns_forward_umma256(U2Ctx& c, int m, int T, float eps, float alph
         u2_store_block(c, v, row, col0, pass < 2 ? u2_block_w(Wimg, ri, ci) : u2_block_w(Xh, ri, ci), pass, false);
       } else {
         // all three buffers are on their way out: the first must have been read before it is rewritten
-        if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        if (umma::leader(tid)) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         __syncthreads();
         u2_store_block(c, v, row, col0, u2_block_w(Xh, ri, ci), 0, true);
       }
@@ -474,7 +474,7 @@ __device__ bool u2_products_dx_dm(U2Ctx& c, int m, int D, const float* dY, const
     if (pass < 3) {
       u2_store_block(c, v, row, col0, dst, pass, false);
     } else {
-      if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // buffer 0 is on its way out
+      if (umma::leader(tid)) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // buffer 0 is on its way out
       __syncthreads();
       u2_store_block(c, v, row, col0, dst, 0, true);
     }

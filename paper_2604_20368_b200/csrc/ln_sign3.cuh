@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(256, 2) k_sign3(const bf16* __restrict__ tok, 
     const uint32_t tacc = tmem_base;
     constexpr uint32_t YB = 2 * GU_KB * D * 2;                       // bytes of one block (hi + lo)
     const bf16* Yh = Yimg + (long long)bh * nkb * (2 * GU_KB * D);
-    if (tid == 0) { umma::mbar_expect_tx(&mbar_y, YB); umma::bulk_load(sY, Yh, YB, &mbar_y); }
+    if (umma::leader(tid)) { umma::mbar_expect_tx(&mbar_y, YB); umma::bulk_load(sY, Yh, YB, &mbar_y); }
     const bf16* Uh = U + (long long)bh * n * D;
     for (int p = tid; p < 128 * (D / 8); p += nthr) {
       const int r = p / (D / 8), c8 = (p % (D / 8)) * 8;
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(256, 2) k_sign3(const bf16* __restrict__ tok, 
     }
     umma::fence_smem_to_mma();
     __syncthreads();
-    if (tid == 0) {
+    if (umma::leader(tid)) {
       const uint32_t idesc = umma::instr_desc(GU_KB, false, false);
       uint32_t ph = 0;
       for (int kb = 0; kb < nkb; ++kb) {

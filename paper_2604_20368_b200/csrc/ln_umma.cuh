@@ -44,7 +44,20 @@ __device__ __forceinline__ uint32_t instr_desc(int N, bool a_mn_major, bool b_mn
          ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// D[tmem] (+)= A * B for one K-step; issued by ONE thread.
+// The one thread of a CTA (of the warp) that issues tensor-core and bulk-copy instructions; the same thread at every call.
+// tcgen05.mma takes its operands from uniform registers.  Behind elect.sync the compiler knows that one lane is active
+// and moves them there directly; behind a test of threadIdx it has to cover the case of several lanes with different
+// operands and wraps every instruction in a loop: 165 to 208 clocks per MMA, whatever its size, against the 9 (N = 16)
+// to 64 (N = 128) the tensor core takes (measured with 4096 MMAs in a row per SM, run-time shapes).  In the kernels,
+// whose loops are unrolled, the step took k_mid_fwd / k_mid_bwd at m = 256 from 923 / 1673 to 886 / 1580 us.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ bool leader(int tid) { return __shfl_sync(0xffffffffu, tid >> 5, 0) == 0 && elect_one(); }
+
+// D[tmem] (+)= A * B for one K-step; issued by ONE thread (see leader()).
 __device__ __forceinline__ void mma(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, bool accumulate) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
                ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate ? 1u : 0u) : "memory");
