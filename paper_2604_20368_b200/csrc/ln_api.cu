@@ -338,6 +338,23 @@ struct TraceScope {
 };
 #define LN_LAUNCH(name, st, ...) do { TraceScope ts_(name, st); __VA_ARGS__; note_launch(); } while (0)
 
+// Every kernel is launched as a programmatic dependent of the one before it on its stream (see pdl_wait in
+// ln_common.cuh): the launch of a kernel overlaps the end of the one before.
+inline cudaLaunchAttribute early_launch() {
+  cudaLaunchAttribute a = {};
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
+}
+template <typename... KArgs, typename... Args>
+void enqueue(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cudaLaunchAttribute at = early_launch();
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
+
 // Side stream.  The per-head kernels (Newton-Schulz and its adjoint: one CTA or cluster per head, bound by the
 // latency of a chain of small products) do not depend on the token-sized kernels next to them, so the entry
 // points enqueue them on a second stream of the library, forked from and joined back into the caller's stream
@@ -437,10 +454,11 @@ template <typename... KArgs, typename... Args>
 void launch_clustered(void (*kern)(KArgs...), int grid, int cl, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cl; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
+  cudaLaunchAttribute at[2];
+  at[0] = early_launch();
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = cl; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 2;
   cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
 
@@ -448,8 +466,8 @@ void launch_clustered(void (*kern)(KArgs...), int grid, int cl, size_t smem, cud
 template <typename T>
 void launch_pool(const ln_problem* p, const T* src, float* L, cudaStream_t st) {
   const int bin_tokens = ((p->gh + p->mh - 1) / p->mh) * ((p->gw + p->mw - 1) / p->mw);
-  if (bin_tokens >= 64) LN_LAUNCH("k_pool", st, k_pool_wide<T><<<dim3(p->m, p->B * p->H), 256, 0, st>>>(src, L, geom_of(p)));
-  else LN_LAUNCH("k_pool", st, k_pool<T><<<dim3(cdiv(p->m, 256 / (p->d / 4)), p->B * p->H), 256, 0, st>>>(src, L, geom_of(p)));
+  if (bin_tokens >= 64) LN_LAUNCH("k_pool", st, enqueue(k_pool_wide<T>, dim3(p->m, p->B * p->H), 256, 0, st, src, L, geom_of(p)));
+  else LN_LAUNCH("k_pool", st, enqueue(k_pool<T>, dim3(cdiv(p->m, 256 / (p->d / 4)), p->B * p->H), 256, 0, st, src, L, geom_of(p)));
 }
 
 template <typename T> constexpr int is_f32() { return std::is_same<T, float>::value ? 1 : 0; }
@@ -476,10 +494,10 @@ void launch_l1_args(const char* name, L1Args& a, int nprob, int batch, cudaStrea
   }
   if (l.qn == 4) {
     want_smem(k_l1<4>, l.smem);
-    LN_LAUNCH(name, st, k_l1<4><<<l.grid, l.block, l.smem, st>>>(a));
+    LN_LAUNCH(name, st, enqueue(k_l1<4>, l.grid, l.block, l.smem, st, a));
   } else {
     want_smem(k_l1<2>, l.smem);
-    LN_LAUNCH(name, st, k_l1<2><<<l.grid, l.block, l.smem, st>>>(a));
+    LN_LAUNCH(name, st, enqueue(k_l1<2>, l.grid, l.block, l.smem, st, a));
   }
 }
 
@@ -510,7 +528,7 @@ int fwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
     launch_pool<T>(p, p->lm_mode == 1 ? K : Q, x.Lf, st);
   } else {
     const long long cnt = (long long)BH * m * D;
-    LN_LAUNCH("k_to_f32", st, k_to_f32<T><<<cdiv(cnt, 256), 256, 0, st>>>(L, x.Lf, cnt));
+    LN_LAUNCH("k_to_f32", st, enqueue(k_to_f32<T>, cdiv(cnt, 256), 256, 0, st, L, x.Lf, cnt));
   }
   // the three kernel blocks: C = k(Q,L) with its row sums, R^T = k(K,L), W = k(L,L)
   // (not for many small heads, where the per-head kernel fills the GPU and the split launches cost more than the
@@ -589,12 +607,12 @@ int fwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
   if constexpr (std::is_same<T, bf16>::value)
   {
     want_smem(k_tn_mma<D>, tn_mma_smem<D>());
-    LN_LAUNCH("tn_M", sm_, k_tn_mma<D><<<dim3(pl.chunks, cdiv(m, 64), BH), 256, tn_mma_smem<D>(), sm_>>>(x.Rt, pl.ldm, nullptr, V, Mdst, nullptr, n, m, pl.rpc));
+    LN_LAUNCH("tn_M", sm_, enqueue(k_tn_mma<D>, dim3(pl.chunks, cdiv(m, 64), BH), 256, tn_mma_smem<D>(), sm_, x.Rt, pl.ldm, nullptr, V, Mdst, nullptr, n, m, pl.rpc));
   }
   else
-    LN_LAUNCH("tn_M", sm_, k_tn<T, D><<<dim3(pl.chunks, cdiv(m, 64), BH), 256, 0, sm_>>>(x.Rt, pl.ldm, nullptr, V, Mdst, nullptr, n, m, pl.rpc));
+    LN_LAUNCH("tn_M", sm_, enqueue(k_tn<T, D>, dim3(pl.chunks, cdiv(m, 64), BH), 256, 0, sm_, x.Rt, pl.ldm, nullptr, V, Mdst, nullptr, n, m, pl.rpc));
   // whitening scale from the statistics the C block left (Eq. 6), before the map is folded
-  if (bw) LN_LAUNCH("k_wstat_final", st, k_wstat_final<<<dim3(cdiv(m, 32), p->H), 256, 0, st>>>(w.stat, p->B, p->H, n, m, pl.l1_tiles, p->whiten_eps,
+  if (bw) LN_LAUNCH("k_wstat_final", st, enqueue(k_wstat_final, dim3(cdiv(m, 32), p->H), 256, 0, st, w.stat, p->B, p->H, n, m, pl.l1_tiles, p->whiten_eps,
                                                                                                p->whiten_batch, x.cbar));
   // Newton-Schulz, Y = X M, folded map
   if (side.on() && !deep) { side.join(st); launch_mid(st, 2); }
@@ -613,18 +631,18 @@ int fwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
     if (epi && epi->src) {
       const size_t smem = nn_umma_stage_dwc<D>() + (size_t)epi->ks * epi->ks * D * sizeof(float);
       want_smem(k_nn_umma<D, true>, smem);
-      LN_LAUNCH("nn_O", st, k_nn_umma<D, true><<<dim3(cdiv(n, 128), BH), 256, smem, st>>>(x.C, pl.ldm, p->map_mode == 1 ? x.mu : nullptr,
+      LN_LAUNCH("nn_O", st, enqueue(k_nn_umma<D, true>, dim3(cdiv(n, 128), BH), 256, smem, st, x.C, pl.ldm, p->map_mode == 1 ? x.mu : nullptr,
                                                                                       reinterpret_cast<const bf16*>(x.Yimg), x.ybar, O, n, m, dev_status, *epi));
     } else {
       const size_t smem = nn_umma_smem<D>();
       want_smem(k_nn_umma<D>, smem);
-      LN_LAUNCH("nn_O", st, k_nn_umma<D><<<dim3(cdiv(n, 128), BH), 256, smem, st>>>(x.C, pl.ldm, p->map_mode == 1 ? x.mu : nullptr,
+      LN_LAUNCH("nn_O", st, enqueue(k_nn_umma<D>, dim3(cdiv(n, 128), BH), 256, smem, st, x.C, pl.ldm, p->map_mode == 1 ? x.mu : nullptr,
                                                                                 reinterpret_cast<const bf16*>(x.Yimg), x.ybar, O, n, m, dev_status, DwcEpi()));
     }
   } else if constexpr (std::is_same<T, bf16>::value)
-    LN_LAUNCH("nn_O", st, k_nn_mma<D><<<dim3(cdiv(n, 64), BH), 256, 0, st>>>(x.C, pl.ldm, p->map_mode == 1 ? x.mu : nullptr, x.Yt, x.ybar, O, n, m));
+    LN_LAUNCH("nn_O", st, enqueue(k_nn_mma<D>, dim3(cdiv(n, 64), BH), 256, 0, st, x.C, pl.ldm, p->map_mode == 1 ? x.mu : nullptr, x.Yt, x.ybar, O, n, m));
   else
-    LN_LAUNCH("nn_O", st, k_nn<T, D><<<dim3(cdiv(n, 64), BH), 256, 0, st>>>(x.C, pl.ldm, p->map_mode == 1 ? x.mu : nullptr, x.Yt, x.ybar, O, n, m));
+    LN_LAUNCH("nn_O", st, enqueue(k_nn<T, D>, dim3(cdiv(n, 64), BH), 256, 0, st, x.C, pl.ldm, p->map_mode == 1 ? x.mu : nullptr, x.Yt, x.ybar, O, n, m));
   return launch_ok();
 }
 
@@ -642,21 +660,21 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
     if constexpr (std::is_same<T, bf16>::value)
     {
       want_smem(k_tn_mma<D>, tn_mma_smem<D>());
-      LN_LAUNCH("tn_dY", s, k_tn_mma<D><<<dim3(ch, cdiv(m, 64), BH), 256, tn_mma_smem<D>(), s>>>(x.C, pl.ldm, mu, dO, w.dYtpart, w.dybpart, n, m, pl.rpc));
+      LN_LAUNCH("tn_dY", s, enqueue(k_tn_mma<D>, dim3(ch, cdiv(m, 64), BH), 256, tn_mma_smem<D>(), s, x.C, pl.ldm, mu, dO, w.dYtpart, w.dybpart, n, m, pl.rpc));
     }
     else
-      LN_LAUNCH("tn_dY", s, k_tn<T, D><<<dim3(ch, cdiv(m, 64), BH), 256, 0, s>>>(x.C, pl.ldm, mu, dO, w.dYtpart, w.dybpart, n, m, pl.rpc));
+      LN_LAUNCH("tn_dY", s, enqueue(k_tn<T, D>, dim3(ch, cdiv(m, 64), BH), 256, 0, s, x.C, pl.ldm, mu, dO, w.dYtpart, w.dybpart, n, m, pl.rpc));
   };
   auto launch_ntg_C = [&]() {
     if constexpr (std::is_same<T, bf16>::value) {
       if constexpr (D == 64 || D == 128) {
         want_smem(k_ntg_umma<D>, ntg_umma_smem<D>());
-        LN_LAUNCH("ntg_C", st, k_ntg_umma<D><<<dim3(cdiv(n, 128), BH), 256, ntg_umma_smem<D>(), st>>>(dO, reinterpret_cast<const bf16*>(x.Yimg), x.C, pl.ldm,
+        LN_LAUNCH("ntg_C", st, enqueue(k_ntg_umma<D>, dim3(cdiv(n, 128), BH), 256, ntg_umma_smem<D>(), st, dO, reinterpret_cast<const bf16*>(x.Yimg), x.C, pl.ldm,
                                                                                                   w.G, n, m, inv_lambda, dev_status));
       } else
-        LN_LAUNCH("ntg_C", st, k_nt_g_mma<D><<<dim3(cdiv(n, 64), cdiv(m, 64), BH), 256, 0, st>>>(dO, x.Yt, x.C, pl.ldm, w.G, n, m, inv_lambda));
+        LN_LAUNCH("ntg_C", st, enqueue(k_nt_g_mma<D>, dim3(cdiv(n, 64), cdiv(m, 64), BH), 256, 0, st, dO, x.Yt, x.C, pl.ldm, w.G, n, m, inv_lambda));
     } else {
-      LN_LAUNCH("ntg_C", st, k_nt_g<T, D><<<dim3(cdiv(n, 64), cdiv(m, 64), BH), 256, 0, st>>>(dO, x.Yt, x.C, pl.ldm, w.G, n, m, inv_lambda));
+      LN_LAUNCH("ntg_C", st, enqueue(k_nt_g<T, D>, dim3(cdiv(n, 64), cdiv(m, 64), BH), 256, 0, st, dO, x.Yt, x.C, pl.ldm, w.G, n, m, inv_lambda));
     }
   };
   const bool fused_sign = pl.s2_chunks > 0;
@@ -678,7 +696,7 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
     if constexpr (std::is_same<T, bf16>::value && (D == 64 || D == 128)) {
       auto go = [&](auto kern) {
         want_smem(kern, sign3_smem_bytes());
-        LN_LAUNCH(name, st, kern<<<dim3(pl.s3_tiles, D / 64, BH), dim3(16, pl.s2_tg), sign3_smem_bytes(), st>>>(
+        LN_LAUNCH(name, st, enqueue(kern, dim3(pl.s3_tiles, D / 64, BH), dim3(16, pl.s2_tg), sign3_smem_bytes(), st,
                       tokp, SBp, Up, reinterpret_cast<const bf16*>(Yimgp), Ap, pl.ldm, rowsp, partp, n, m, inv_lambda, dev_status, kap, p->H));
       };
       using TO = std::remove_pointer_t<decltype(rowsp)>;
@@ -713,12 +731,12 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
     if constexpr (std::is_same<T, bf16>::value) {
       if constexpr (D == 64 || D == 128) {
         want_smem(k_ntg_umma<D>, ntg_umma_smem<D>());
-        LN_LAUNCH("ntg_R", s, k_ntg_umma<D><<<dim3(cdiv(n, 128), BH), 256, ntg_umma_smem<D>(), s>>>(V, reinterpret_cast<const bf16*>(w.dMimg), x.Rt, pl.ldm,
+        LN_LAUNCH("ntg_R", s, enqueue(k_ntg_umma<D>, dim3(cdiv(n, 128), BH), 256, ntg_umma_smem<D>(), s, V, reinterpret_cast<const bf16*>(w.dMimg), x.Rt, pl.ldm,
                                                                                                 w.G2, n, m, inv_lambda, dev_status));
       } else
-        LN_LAUNCH("ntg_R", s, k_nt_g_mma<D><<<dim3(cdiv(n, 64), cdiv(m, 64), BH), 256, 0, s>>>(V, w.dM, x.Rt, pl.ldm, w.G2, n, m, inv_lambda));
+        LN_LAUNCH("ntg_R", s, enqueue(k_nt_g_mma<D>, dim3(cdiv(n, 64), cdiv(m, 64), BH), 256, 0, s, V, w.dM, x.Rt, pl.ldm, w.G2, n, m, inv_lambda));
     } else {
-      LN_LAUNCH("ntg_R", s, k_nt_g<T, D><<<dim3(cdiv(n, 64), cdiv(m, 64), BH), 256, 0, s>>>(V, w.dM, x.Rt, pl.ldm, w.G2, n, m, inv_lambda));
+      LN_LAUNCH("ntg_R", s, enqueue(k_nt_g<T, D>, dim3(cdiv(n, 64), cdiv(m, 64), BH), 256, 0, s, V, w.dM, x.Rt, pl.ldm, w.G2, n, m, inv_lambda));
     }
   };
   auto launch_nn_dV = [&](cudaStream_t s) {
@@ -727,24 +745,24 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
         if (epi && epi->src) {
           const size_t smem = nn_umma_stage_dwc<D>() + (size_t)epi->ks * epi->ks * D * sizeof(float);
           want_smem(k_nn_umma<D, true>, smem);
-          LN_LAUNCH("nn_dV", s, k_nn_umma<D, true><<<dim3(cdiv(n, 128), BH), 256, smem, s>>>(x.Rt, pl.ldm, nullptr, reinterpret_cast<const bf16*>(w.dMimg),
+          LN_LAUNCH("nn_dV", s, enqueue(k_nn_umma<D, true>, dim3(cdiv(n, 128), BH), 256, smem, s, x.Rt, pl.ldm, nullptr, reinterpret_cast<const bf16*>(w.dMimg),
                                                                                          nullptr, dV, n, m, dev_status, *epi));
         } else {
           const size_t smem = nn_umma_smem<D>();
           want_smem(k_nn_umma<D>, smem);
-          LN_LAUNCH("nn_dV", s, k_nn_umma<D><<<dim3(cdiv(n, 128), BH), 256, smem, s>>>(x.Rt, pl.ldm, nullptr, reinterpret_cast<const bf16*>(w.dMimg),
+          LN_LAUNCH("nn_dV", s, enqueue(k_nn_umma<D>, dim3(cdiv(n, 128), BH), 256, smem, s, x.Rt, pl.ldm, nullptr, reinterpret_cast<const bf16*>(w.dMimg),
                                                                                    nullptr, dV, n, m, dev_status, DwcEpi()));
         }
       } else
-        LN_LAUNCH("nn_dV", s, k_nn_mma<D><<<dim3(cdiv(n, 64), BH), 256, 0, s>>>(x.Rt, pl.ldm, nullptr, w.dM, nullptr, dV, n, m));
+        LN_LAUNCH("nn_dV", s, enqueue(k_nn_mma<D>, dim3(cdiv(n, 64), BH), 256, 0, s, x.Rt, pl.ldm, nullptr, w.dM, nullptr, dV, n, m));
     } else {
-      LN_LAUNCH("nn_dV", s, k_nn<T, D><<<dim3(cdiv(n, 64), BH), 256, 0, s>>>(x.Rt, pl.ldm, nullptr, w.dM, nullptr, dV, n, m));
+      LN_LAUNCH("nn_dV", s, enqueue(k_nn<T, D>, dim3(cdiv(n, 64), BH), 256, 0, s, x.Rt, pl.ldm, nullptr, w.dM, nullptr, dV, n, m));
     }
   };
   auto launch_sign_W = [&](cudaStream_t s) {
     // one set: GW is symmetrised, so the row pass carries both roles of L.  Two sets: rows -> pooled queries, columns -> pooled keys
-    LN_LAUNCH("sign_rows_dLW", s, k_sign_rows<float, float, float, D><<<dim3(cdiv(m, 64), BH), 256, 0, s>>>(LfR, LfC, w.GW, pl.ldm, w.dLW, m, m));
-    if (two) LN_LAUNCH("sign_cols_dLW", s, k_sign_cols<float, float, D><<<dim3(1, cdiv(m, 64), BH), 256, 0, s>>>(LfR, LfC, w.GW, pl.ldm, w.dLW2, m, m, (m + 31) / 32 * 32));
+    LN_LAUNCH("sign_rows_dLW", s, enqueue(k_sign_rows<float, float, float, D>, dim3(cdiv(m, 64), BH), 256, 0, s, LfR, LfC, w.GW, pl.ldm, w.dLW, m, m, 0, nullptr, 1.f));
+    if (two) LN_LAUNCH("sign_cols_dLW", s, enqueue(k_sign_cols<float, float, D>, dim3(1, cdiv(m, 64), BH), 256, 0, s, LfR, LfC, w.GW, pl.ldm, w.dLW2, m, m, (m + 31) / 32 * 32, nullptr, 1.f));
   };
   // Side stream: the per-head kernel, the landmark-block sign pass and dV (bound by latency and by memory) run beside
   // the sign passes (bound by arithmetic).  The upstream of the key-side block, which the second sign pass waits for,
@@ -763,7 +781,7 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
   // Batch-statistic whitening: ds needs Z'^T dO of every batch element of a head, and the query-side sign pass needs
   // the coefficient it gives, so Z'^T dO stays on the caller's stream in front of both.
   const float* const kap = bw ? w.kap : nullptr;
-  if (bw) LN_LAUNCH("k_whiten_bwd", st, k_whiten_bwd<<<dim3(cdiv(m, 8), p->H), 256, 0, st>>>(x.Y, w.dYtpart, ch, p->whiten_batch, x.cbar, p->B, p->H,
+  if (bw) LN_LAUNCH("k_whiten_bwd", st, enqueue(k_whiten_bwd, dim3(cdiv(m, 8), p->H), 256, 0, st, x.Y, w.dYtpart, ch, p->whiten_batch, x.cbar, p->B, p->H,
                                                                                             n, m, D, w.kap));
   if (side.on()) {
     side.fork(st);
@@ -780,19 +798,19 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
   }
   if (sign3) {
     const long long cnt = (long long)BH * m * D;
-    LN_LAUNCH("k_fold_landmarks", st, k_fold_landmarks<<<cdiv(cnt, 256), 256, 0, st>>>(LfC, w.SB, D, cnt));
-    if (two) LN_LAUNCH("k_fold_landmarks", st, k_fold_landmarks<<<cdiv(cnt, 256), 256, 0, st>>>(LfR, w.SBq, D, cnt));
+    LN_LAUNCH("k_fold_landmarks", st, enqueue(k_fold_landmarks, cdiv(cnt, 256), 256, 0, st, LfC, w.SB, D, cnt));
+    if (two) LN_LAUNCH("k_fold_landmarks", st, enqueue(k_fold_landmarks, cdiv(cnt, 256), 256, 0, st, LfR, w.SBq, D, cnt));
     if (qrows_f) launch_sign3("sign3_dQ_dLC", Q, dO, x.Yimg, x.C, qrows_f, w.dLCpart, w.SB, kap);
     else launch_sign3("sign3_dQ_dLC", Q, dO, x.Yimg, x.C, dQ, w.dLCpart, w.SB, kap);
   } else {
     launch_ntg_C();
-    if (bw) LN_LAUNCH("k_g_whiten_add", st, k_g_whiten_add<<<dim3(cdiv((long long)n * pl.ldm, 256), BH), 256, 0, st>>>(w.G, x.C, w.kap, p->H, n, m, pl.ldm, inv_lambda));
+    if (bw) LN_LAUNCH("k_g_whiten_add", st, enqueue(k_g_whiten_add, dim3(cdiv((long long)n * pl.ldm, 256), BH), 256, 0, st, w.G, x.C, w.kap, p->H, n, m, pl.ldm, inv_lambda));
   }
   if (sign3) {
   } else if (fused_sign) {
     auto launch2 = [&](const char* name, auto kern, const T* tokp, auto* rowsp, float* partp) {
       want_smem(kern, pl.s2_smem);
-      LN_LAUNCH(name, st, kern<<<dim3(chq, D / 64, BH), dim3(16, pl.s2_tg), pl.s2_smem, st>>>(tokp, x.Lf, w.G, pl.ldm, rowsp, partp, n, m, D, pl.s2q_rpc));
+      LN_LAUNCH(name, st, enqueue(kern, dim3(chq, D / 64, BH), dim3(16, pl.s2_tg), pl.s2_smem, st, tokp, x.Lf, w.G, pl.ldm, rowsp, partp, n, m, D, pl.s2q_rpc));
     };
     if (poolQ) {
       if (pl.s2_tg == S2_TGMAX) launch2("sign2_dQ_dLC", k_sign2<T, float, 1>, Q, w.dKpart, w.dLCpart);
@@ -802,9 +820,9 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
       else launch2("sign2_dQ_dLC", k_sign2<T, T, 2>, Q, dQ, w.dLCpart);
     }
   } else {
-    if (qrows_f) LN_LAUNCH("sign_rows_dQ", st, k_sign_rows<T, float, float, D><<<dim3(cdiv(n, 64), BH), 256, 0, st>>>(Q, LfC, w.G, pl.ldm, qrows_f, n, m));
-    else LN_LAUNCH("sign_rows_dQ", st, k_sign_rows<T, float, T, D><<<dim3(cdiv(n, 64), BH), 256, 0, st>>>(Q, LfC, w.G, pl.ldm, dQ, n, m));
-    LN_LAUNCH("sign_cols_dLC", st, k_sign_cols<T, float, D><<<dim3(ch, cdiv(m, 64), BH), 256, 0, st>>>(Q, LfC, w.G, pl.ldm, w.dLCpart, n, m, pl.rpc));
+    if (qrows_f) LN_LAUNCH("sign_rows_dQ", st, enqueue(k_sign_rows<T, float, float, D>, dim3(cdiv(n, 64), BH), 256, 0, st, Q, LfC, w.G, pl.ldm, qrows_f, n, m, 0, nullptr, 1.f));
+    else LN_LAUNCH("sign_rows_dQ", st, enqueue(k_sign_rows<T, float, T, D>, dim3(cdiv(n, 64), BH), 256, 0, st, Q, LfC, w.G, pl.ldm, dQ, n, m, 0, nullptr, 1.f));
+    LN_LAUNCH("sign_cols_dLC", st, enqueue(k_sign_cols<T, float, D>, dim3(ch, cdiv(m, 64), BH), 256, 0, st, Q, LfC, w.G, pl.ldm, w.dLCpart, n, m, pl.rpc, nullptr, 1.f));
   }
   if (side.on()) { side.join_mark(st); if (!ntg_on_side && !sign3) launch_ntg_R(st); }
   else { launch_mid(st); launch_sign_W(st); if (!sign3) launch_ntg_R(st); launch_nn_dV(st); }
@@ -815,7 +833,7 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
   } else if (fused_sign) {
     auto launch2 = [&](const char* name, auto kern, const T* tokp, auto* rowsp, float* partp) {
       want_smem(kern, pl.s2_smem);
-      LN_LAUNCH(name, st, kern<<<dim3(chs, D / 64, BH), dim3(16, pl.s2_tg), pl.s2_smem, st>>>(tokp, x.Lf, w.G2, pl.ldm, rowsp, partp, n, m, D, pl.s2_rpc));
+      LN_LAUNCH(name, st, enqueue(kern, dim3(chs, D / 64, BH), dim3(16, pl.s2_tg), pl.s2_smem, st, tokp, x.Lf, w.G2, pl.ldm, rowsp, partp, n, m, D, pl.s2_rpc));
     };
     if (poolQ) {
       if (pl.s2_tg == S2_TGMAX) launch2("sign2_dK_dLR", k_sign2<T, T, 1>, K, dK, w.dLRpart);
@@ -825,22 +843,22 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
       else launch2("sign2_dK_dLR", k_sign2<T, float, 2>, K, w.dKpart, w.dLRpart);
     }
   } else {
-    if (!krows_f) LN_LAUNCH("sign_rows_dK", st, k_sign_rows<T, float, T, D><<<dim3(cdiv(n, 64), BH), 256, 0, st>>>(K, LfR, w.G2, pl.ldm, dK, n, m));
-    else LN_LAUNCH("sign_rows_dK", st, k_sign_rows<T, float, float, D><<<dim3(cdiv(n, 64), BH), 256, 0, st>>>(K, LfR, w.G2, pl.ldm, krows_f, n, m));
-    LN_LAUNCH("sign_cols_dLR", st, k_sign_cols<T, float, D><<<dim3(ch, cdiv(m, 64), BH), 256, 0, st>>>(K, LfR, w.G2, pl.ldm, w.dLRpart, n, m, pl.rpc));
+    if (!krows_f) LN_LAUNCH("sign_rows_dK", st, enqueue(k_sign_rows<T, float, T, D>, dim3(cdiv(n, 64), BH), 256, 0, st, K, LfR, w.G2, pl.ldm, dK, n, m, 0, nullptr, 1.f));
+    else LN_LAUNCH("sign_rows_dK", st, enqueue(k_sign_rows<T, float, float, D>, dim3(cdiv(n, 64), BH), 256, 0, st, K, LfR, w.G2, pl.ldm, krows_f, n, m, 0, nullptr, 1.f));
+    LN_LAUNCH("sign_cols_dLR", st, enqueue(k_sign_cols<T, float, D>, dim3(ch, cdiv(m, 64), BH), 256, 0, st, K, LfR, w.G2, pl.ldm, w.dLRpart, n, m, pl.rpc, nullptr, 1.f));
   }
   // landmark gradient and its way back to the keys
   if (side.on()) side.join(st);      // dV and the landmark-block part are complete
   const int md = m * D;
   if (two) {                  // pooled keys: columns of C and of W; pooled queries: columns of R^T and rows of W
-    LN_LAUNCH("k_reduce3", st, k_reduce3_wide<float><<<dim3(cdiv(md, 128), BH), 256, 0, st>>>(w.dLCpart, chq, w.dLW2, 1, nullptr, 0, w.dLtot, md));
-    LN_LAUNCH("k_reduce3", st, k_reduce3_wide<float><<<dim3(cdiv(md, 128), BH), 256, 0, st>>>(w.dLRpart, chs, w.dLW, 1, nullptr, 0, w.dLqtot, md));
-    LN_LAUNCH("k_pool_bwd", st, k_pool_bwd<T><<<dim3(cdiv((long long)n * (D / 4), 256 * POOL_EPT), BH), 256, 0, st>>>(w.dKpart, w.dLtot, dK, geom_of(p), 1));
-    LN_LAUNCH("k_pool_bwd", st, k_pool_bwd<T><<<dim3(cdiv((long long)n * (D / 4), 256 * POOL_EPT), BH), 256, 0, st>>>(w.dQpart, w.dLqtot, dQ, geom_of(p), 1));
+    LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3_wide<float>, dim3(cdiv(md, 128), BH), 256, 0, st, w.dLCpart, chq, w.dLW2, 1, nullptr, 0, w.dLtot, md));
+    LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3_wide<float>, dim3(cdiv(md, 128), BH), 256, 0, st, w.dLRpart, chs, w.dLW, 1, nullptr, 0, w.dLqtot, md));
+    LN_LAUNCH("k_pool_bwd", st, enqueue(k_pool_bwd<T>, dim3(cdiv((long long)n * (D / 4), 256 * POOL_EPT), BH), 256, 0, st, w.dKpart, w.dLtot, dK, geom_of(p), 1));
+    LN_LAUNCH("k_pool_bwd", st, enqueue(k_pool_bwd<T>, dim3(cdiv((long long)n * (D / 4), 256 * POOL_EPT), BH), 256, 0, st, w.dQpart, w.dLqtot, dQ, geom_of(p), 1));
   } else if (p->lm_mode >= 1) {      // the landmark gradient returns to the pooled tensor (keys, or queries for lm_mode 2)
-    if (chq + chs >= 16) LN_LAUNCH("k_reduce3", st, k_reduce3_wide<float><<<dim3(cdiv(md, 128), BH), 256, 0, st>>>(w.dLCpart, chq, w.dLRpart, chs, w.dLW, 1, w.dLtot, md));
-    else LN_LAUNCH("k_reduce3", st, k_reduce3<float><<<dim3(cdiv(md, 1024), BH), 256, 0, st>>>(w.dLCpart, chq, w.dLRpart, chs, w.dLW, 1, w.dLtot, md));
-    LN_LAUNCH("k_pool_bwd", st, k_pool_bwd<T><<<dim3(cdiv((long long)n * (D / 4), 256 * POOL_EPT), BH), 256, 0, st>>>(w.dKpart, w.dLtot, poolQ ? dQ : dK, geom_of(p), 1));
+    if (chq + chs >= 16) LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3_wide<float>, dim3(cdiv(md, 128), BH), 256, 0, st, w.dLCpart, chq, w.dLRpart, chs, w.dLW, 1, w.dLtot, md));
+    else LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3<float>, dim3(cdiv(md, 1024), BH), 256, 0, st, w.dLCpart, chq, w.dLRpart, chs, w.dLW, 1, w.dLtot, md));
+    LN_LAUNCH("k_pool_bwd", st, enqueue(k_pool_bwd<T>, dim3(cdiv((long long)n * (D / 4), 256 * POOL_EPT), BH), 256, 0, st, w.dKpart, w.dLtot, poolQ ? dQ : dK, geom_of(p), 1));
     if (p->lm_filter) {          // gradient of the selection filter, summed over the batch elements of a head
       const int taps = (p->gh / p->mh) * (p->gw / p->mw);
       // the (batch element, landmark) pairs are split over enough CTAs to fill the GPU; the partial sums go to the query-side
@@ -852,16 +870,16 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
       if (splits > 65535) splits = 65535;
       if (splits < 1) splits = 1;
       float* fpart = splits > 1 ? w.dLCpart : p->lm_filter_grad;
-      LN_LAUNCH("k_filter_grad", st, k_filter_grad<T><<<dim3(taps, p->H, (unsigned)splits), 256, 0, st>>>(poolQ ? Q : K, w.dLtot, fpart, geom_of(p), p->B));
+      LN_LAUNCH("k_filter_grad", st, enqueue(k_filter_grad<T>, dim3(taps, p->H, (unsigned)splits), 256, 0, st, poolQ ? Q : K, w.dLtot, fpart, geom_of(p), p->B));
       if (splits > 1) {
         const int count = p->H * taps * D;
-        LN_LAUNCH("k_filter_reduce", st, k_filter_reduce<<<cdiv(count, 1024), 256, 0, st>>>(w.dLCpart, (int)splits, p->lm_filter_grad, count));
+        LN_LAUNCH("k_filter_reduce", st, enqueue(k_filter_reduce, cdiv(count, 1024), 256, 0, st, w.dLCpart, (int)splits, p->lm_filter_grad, count));
       }
     }
   } else {
-    if (chq + chs >= 16) LN_LAUNCH("k_reduce3", st, k_reduce3_wide<T><<<dim3(cdiv(md, 128), BH), 256, 0, st>>>(w.dLCpart, chq, w.dLRpart, chs, w.dLW, 1, dL, md));
-    else LN_LAUNCH("k_reduce3", st, k_reduce3<T><<<dim3(cdiv(md, 1024), BH), 256, 0, st>>>(w.dLCpart, chq, w.dLRpart, chs, w.dLW, 1, dL, md));
-    LN_LAUNCH("k_pool_bwd", st, k_pool_bwd<T><<<dim3(cdiv((long long)n * (D / 4), 256 * POOL_EPT), BH), 256, 0, st>>>(w.dKpart, nullptr, dK, geom_of(p), 0));
+    if (chq + chs >= 16) LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3_wide<T>, dim3(cdiv(md, 128), BH), 256, 0, st, w.dLCpart, chq, w.dLRpart, chs, w.dLW, 1, dL, md));
+    else LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3<T>, dim3(cdiv(md, 1024), BH), 256, 0, st, w.dLCpart, chq, w.dLRpart, chs, w.dLW, 1, dL, md));
+    LN_LAUNCH("k_pool_bwd", st, enqueue(k_pool_bwd<T>, dim3(cdiv((long long)n * (D / 4), 256 * POOL_EPT), BH), 256, 0, st, w.dKpart, nullptr, dK, geom_of(p), 0));
   }
   return launch_ok();
 }
@@ -944,13 +962,13 @@ void l1_bwd_impl(int batch, int na, int nb, const T* A, const T* Bm, float lambd
   // the factor dK o K / lambda is formed where the two passes load their tiles of it
   const float il = 1.f / lambda;
   if (w.lsplits > 1) {
-    LN_LAUNCH("k_sign_rows", st, k_sign_rows<T, T, float, D><<<dim3(cdiv(na, 64), batch, w.lsplits), 256, 0, st>>>(A, Bm, dK, nb, w.rowpart, na, nb, w.lper, Kmat, il));
-    LN_LAUNCH("k_reduce3", st, k_reduce3<T><<<dim3(cdiv(na * D, 1024), batch), 256, 0, st>>>(w.rowpart, w.lsplits, nullptr, 0, nullptr, 0, dA, na * D));
+    LN_LAUNCH("k_sign_rows", st, enqueue(k_sign_rows<T, T, float, D>, dim3(cdiv(na, 64), batch, w.lsplits), 256, 0, st, A, Bm, dK, nb, w.rowpart, na, nb, w.lper, Kmat, il));
+    LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3<T>, dim3(cdiv(na * D, 1024), batch), 256, 0, st, w.rowpart, w.lsplits, nullptr, 0, nullptr, 0, dA, na * D));
   } else {
-    LN_LAUNCH("k_sign_rows", st, k_sign_rows<T, T, T, D><<<dim3(cdiv(na, 64), batch), 256, 0, st>>>(A, Bm, dK, nb, dA, na, nb, 0, Kmat, il));
+    LN_LAUNCH("k_sign_rows", st, enqueue(k_sign_rows<T, T, T, D>, dim3(cdiv(na, 64), batch), 256, 0, st, A, Bm, dK, nb, dA, na, nb, 0, Kmat, il));
   }
-  LN_LAUNCH("k_sign_cols", st, k_sign_cols<T, T, D><<<dim3(w.chunks, cdiv(nb, 64), batch), 256, 0, st>>>(A, Bm, dK, nb, w.part, na, nb, w.rpc, Kmat, il));
-  LN_LAUNCH("k_reduce3", st, k_reduce3<T><<<dim3(cdiv(nb * D, 1024), batch), 256, 0, st>>>(w.part, w.chunks, nullptr, 0, nullptr, 0, dB, nb * D));
+  LN_LAUNCH("k_sign_cols", st, enqueue(k_sign_cols<T, T, D>, dim3(w.chunks, cdiv(nb, 64), batch), 256, 0, st, A, Bm, dK, nb, w.part, na, nb, w.rpc, Kmat, il));
+  LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3<T>, dim3(cdiv(nb * D, 1024), batch), 256, 0, st, w.part, w.chunks, nullptr, 0, nullptr, 0, dB, nb * D));
 }
 }  // namespace
 
@@ -1121,8 +1139,8 @@ int laplace_nystrom_whiten_stats(const ln_problem* p, const void* saved, float e
   int sp, rps; wstat_plan(p, &sp, &rps);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   double* part = static_cast<double*>(ws);
-  LN_LAUNCH("k_wstat_part", st, k_wstat_part<<<dim3(sp, pl.BH), 256, 0, st>>>(x.C, pl.ldm, p->n, p->m, rps, part));
-  LN_LAUNCH("k_wstat_final", st, k_wstat_final<<<dim3(cdiv(p->m, 32), p->H), 256, 0, st>>>(part, p->B, p->H, p->n, p->m, sp, eps_w, whiten_out, nullptr));
+  LN_LAUNCH("k_wstat_part", st, enqueue(k_wstat_part, dim3(sp, pl.BH), 256, 0, st, x.C, pl.ldm, p->n, p->m, rps, part));
+  LN_LAUNCH("k_wstat_final", st, enqueue(k_wstat_final, dim3(cdiv(p->m, 32), p->H), 256, 0, st, part, p->B, p->H, p->n, p->m, sp, eps_w, whiten_out, nullptr));
   return launch_ok();
 }
 
@@ -1341,8 +1359,8 @@ int landmarks_pool_bwd(const ln_problem* p, const float* dL, void* dK, void* str
   if (p->lm_mode < 1 || !dL || !dK || !aligned16(dL) || !aligned16(dK)) return LN_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   dim3 grid(cdiv((long long)p->n * (p->d / 4), 256 * POOL_EPT), p->B * p->H);
-  if (p->dtype == LN_F32) LN_LAUNCH("k_pool_bwd", st, k_pool_bwd<float><<<grid, 256, 0, st>>>(nullptr, dL, (float*)dK, geom_of(p), 1));
-  else LN_LAUNCH("k_pool_bwd", st, k_pool_bwd<bf16><<<grid, 256, 0, st>>>(nullptr, dL, (bf16*)dK, geom_of(p), 1));
+  if (p->dtype == LN_F32) LN_LAUNCH("k_pool_bwd", st, enqueue(k_pool_bwd<float>, grid, 256, 0, st, nullptr, dL, (float*)dK, geom_of(p), 1));
+  else LN_LAUNCH("k_pool_bwd", st, enqueue(k_pool_bwd<bf16>, grid, 256, 0, st, nullptr, dL, (bf16*)dK, geom_of(p), 1));
   return launch_ok();
 }
 
@@ -1373,14 +1391,14 @@ int laplace_nystrom_saved_array(const ln_problem* p, const char* name, int64_t i
 int ln_selftest_wait_timeout(int32_t probes, int32_t* dev_status, void* stream) {
   if (probes <= 0 || probes > (1 << 22) || !dev_status) return LN_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  LN_LAUNCH("k_selftest_wait", st, k_selftest_wait<<<1, 32, 0, st>>>(probes, dev_status));
+  LN_LAUNCH("k_selftest_wait", st, enqueue(k_selftest_wait, 1, 32, 0, st, probes, dev_status));
   return launch_ok();
 }
 
 int ln_fp32_add_probe(int32_t blocks, int32_t iters, int32_t mode, float* sink, void* stream) {
   if (blocks <= 0 || iters <= 0 || !sink || mode < 0 || mode > 5) return LN_ERR_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  LN_LAUNCH("k_fp32_add_probe", st, k_fp32_add_probe<<<blocks, 256, 0, st>>>(iters, mode, sink));
+  LN_LAUNCH("k_fp32_add_probe", st, enqueue(k_fp32_add_probe, blocks, 256, 0, st, iters, mode, sink));
   return launch_ok();
 }
 int64_t ln_fp32_add_probe_lane_ops(int32_t blocks, int32_t iters, int32_t mode) {
@@ -1411,7 +1429,7 @@ int dwc_chunks(const ln_problem* p) { const int t = dwc_tokens_per_chunk(p); ret
 size_t rope_table_bytes(const ln_problem* p) { return align_up((size_t)p->gh * p->gw * (p->d / 2) * sizeof(double2), 256); }
 void launch_rope_table(const ln_problem* p, const ln_block* b, double2* tab, cudaStream_t st) {
   const long long cnt = (long long)p->gh * p->gw * (p->d / 2);
-  LN_LAUNCH("rope_table", st, k_rope_table<<<cdiv(cnt, 256), 256, 0, st>>>(tab, cnt, p->d, log2((double)b->rope_base)));
+  LN_LAUNCH("rope_table", st, enqueue(k_rope_table, cdiv(cnt, 256), 256, 0, st, tab, cnt, p->d, log2((double)b->rope_base)));
 }
 template <typename T>
 void launch_rope(const char* name, const ln_problem* p, const double2* tab, const void* X, void* out, double sign, cudaStream_t st) {
@@ -1419,13 +1437,13 @@ void launch_rope(const char* name, const ln_problem* p, const double2* tab, cons
   const int BH = p->B * p->H, gx = (int)cdiv((long long)p->n * (p->d / 4), 256);
   int gy = (int)cdiv(4ll * sm_count(), gx); if (gy > BH) gy = BH; if (gy < 1) gy = 1;
   const int hpc = (BH + gy - 1) / gy; gy = (BH + hpc - 1) / hpc;
-  LN_LAUNCH(name, st, k_rope<T><<<dim3(gx, gy), 256, 0, st>>>((const T*)X, (T*)out, BH, hpc, p->n, p->d, p->prefix, tab, sign));
+  LN_LAUNCH(name, st, enqueue(k_rope<T>, dim3(gx, gy), 256, 0, st, (const T*)X, (T*)out, BH, hpc, p->n, p->d, p->prefix, tab, sign));
 }
 // the tcgen05 product kernels (bf16 storage, 64 or 128 dims) take the convolution branch into their epilogue
 inline bool dwc_in_epilogue(const ln_problem* p) { return p->dtype == LN_BF16 && (p->d == 64 || p->d == 128); }
 template <typename T>
 void launch_dwc_add(const char* name, const ln_problem* p, const ln_block* b, const void* src, void* out, int flip, cudaStream_t st) {
-  LN_LAUNCH(name, st, k_dwc_add<T><<<dim3(cdiv((long long)p->gh * p->gw * (p->d / 4), 256), p->B * p->H), 256, 0, st>>>(
+  LN_LAUNCH(name, st, enqueue(k_dwc_add<T>, dim3(cdiv((long long)p->gh * p->gw * (p->d / 4), 256), p->B * p->H), 256, 0, st,
                 (const T*)src, b->dwc_w, (T*)out, p->H, p->n, p->d, p->prefix, p->gh, p->gw, b->dwc_ks, flip));
 }
 }  // namespace
@@ -1511,21 +1529,21 @@ int laplace_attention_block_bwd(const ln_problem* p, const ln_block* b, const vo
     if (p->dtype == LN_F32) {
       launch_dwc_add<float>("dwc_dV", p, b, dO, dV, 1, st);
       if (b->dwc_ks == 3)
-        LN_LAUNCH("dwc_wgrad", st, k_dwc_wgrad3<float><<<dim3(ch, BH), 256, 0, st>>>((const float*)V, (const float*)dO, wpart, p->n, p->d, p->prefix,
+        LN_LAUNCH("dwc_wgrad", st, enqueue(k_dwc_wgrad3<float>, dim3(ch, BH), 256, 0, st, (const float*)V, (const float*)dO, wpart, p->n, p->d, p->prefix,
                                                                                      p->gh, p->gw, dwc_tokens_per_chunk(p)));
       else
-      LN_LAUNCH("dwc_wgrad", st, k_dwc_wgrad<float><<<dim3(ch, BH, b->dwc_ks), 256, 0, st>>>((const float*)V, (const float*)dO, wpart, p->n, p->d, p->prefix,
+      LN_LAUNCH("dwc_wgrad", st, enqueue(k_dwc_wgrad<float>, dim3(ch, BH, b->dwc_ks), 256, 0, st, (const float*)V, (const float*)dO, wpart, p->n, p->d, p->prefix,
                                                                                             p->gh, p->gw, b->dwc_ks, dwc_tokens_per_chunk(p)));
     } else {
       if (!fused_dwc) launch_dwc_add<bf16>("dwc_dV", p, b, dO, dV, 1, st);
       if (b->dwc_ks == 3)
-        LN_LAUNCH("dwc_wgrad", st, k_dwc_wgrad3<bf16><<<dim3(ch, BH), 256, 0, st>>>((const bf16*)V, (const bf16*)dO, wpart, p->n, p->d, p->prefix,
+        LN_LAUNCH("dwc_wgrad", st, enqueue(k_dwc_wgrad3<bf16>, dim3(ch, BH), 256, 0, st, (const bf16*)V, (const bf16*)dO, wpart, p->n, p->d, p->prefix,
                                                                                     p->gh, p->gw, dwc_tokens_per_chunk(p)));
       else
-      LN_LAUNCH("dwc_wgrad", st, k_dwc_wgrad<bf16><<<dim3(ch, BH, b->dwc_ks), 256, 0, st>>>((const bf16*)V, (const bf16*)dO, wpart, p->n, p->d, p->prefix,
+      LN_LAUNCH("dwc_wgrad", st, enqueue(k_dwc_wgrad<bf16>, dim3(ch, BH, b->dwc_ks), 256, 0, st, (const bf16*)V, (const bf16*)dO, wpart, p->n, p->d, p->prefix,
                                                                                            p->gh, p->gw, b->dwc_ks, dwc_tokens_per_chunk(p)));
     }
-    LN_LAUNCH("dwc_wreduce", st, k_dwc_wreduce<<<dim3(cdiv(cnt, 128), p->H), 256, 0, st>>>(wpart, dWd, p->B, p->H, ch, cnt));
+    LN_LAUNCH("dwc_wreduce", st, enqueue(k_dwc_wreduce, dim3(cdiv(cnt, 128), p->H), 256, 0, st, wpart, dWd, p->B, p->H, ch, cnt));
   }
   return launch_ok();
 }
@@ -1542,7 +1560,7 @@ int laplace_exact_fwd(int32_t batch, int32_t n, int32_t d, int32_t dtype, float 
   auto go = [&](auto kern, size_t smem) {
     want_smem(kern, smem);
     using TT = std::remove_const_t<std::remove_pointer_t<decltype(arg0(kern))>>;
-    LN_LAUNCH("k_exact_fwd", st, kern<<<dim3(cdiv(n, 64), batch), 256, smem, st>>>((const TT*)Q, (const TT*)K, (const TT*)V, (TT*)O, n, nscale, map_mode));
+    LN_LAUNCH("k_exact_fwd", st, enqueue(kern, dim3(cdiv(n, 64), batch), 256, smem, st, (const TT*)Q, (const TT*)K, (const TT*)V, (TT*)O, n, nscale, map_mode));
   };
   if (dtype == LN_F32) { if (d == 32) go(k_exact_fwd<float, 32>, exact_smem_bytes<32>()); else if (d == 64) go(k_exact_fwd<float, 64>, exact_smem_bytes<64>()); else go(k_exact_fwd<float, 128>, exact_smem_bytes<128>()); }
   else { if (d == 32) go(k_exact_fwd<bf16, 32>, exact_smem_bytes<32>()); else if (d == 64) go(k_exact_fwd<bf16, 64>, exact_smem_bytes<64>()); else go(k_exact_fwd<bf16, 128>, exact_smem_bytes<128>()); }

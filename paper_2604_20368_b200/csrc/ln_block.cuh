@@ -20,6 +20,7 @@ template <> __device__ __forceinline__ bf16 from_d<bf16>(double x) { return __do
 // d / 2 channel pairs.  Every head and batch element of a call turns by the same angles, so the double-precision
 // sine and cosine are formed once per (position, pair) instead of once per element.
 __global__ void __launch_bounds__(256) k_rope_table(double2* __restrict__ tab, long long count, int d, double log2_base) {
+  pdl_wait();
   const long long e = (long long)blockIdx.x * 256 + threadIdx.x;
   if (e >= count) return;
   const int i = (int)(e % (d / 2));
@@ -34,6 +35,7 @@ __global__ void __launch_bounds__(256) k_rope_table(double2* __restrict__ tab, l
 template <typename T>
 __global__ void __launch_bounds__(256) k_rope(const T* __restrict__ X, T* __restrict__ out, int BH, int hpc, int n, int d,
                                              int prefix, const double2* __restrict__ tab, double sign) {
+  pdl_wait();
   const int e = blockIdx.x * 256 + threadIdx.x, quads = d / 4;
   if (e >= n * quads) return;
   const int t = e / quads, c = (e % quads) * 4;
@@ -70,6 +72,7 @@ __global__ void __launch_bounds__(256) k_rope(const T* __restrict__ X, T* __rest
 template <typename T>
 __global__ void __launch_bounds__(256) k_dwc_add(const T* __restrict__ src, const float* __restrict__ w, T* __restrict__ out,
                                                 int H, int n, int d, int prefix, int gh, int gw, int ks, int flip) {
+  pdl_wait();
   const int bh = blockIdx.y, h = bh % H, quads = d / 4, half = ks / 2;
   const long long e = (long long)blockIdx.x * 256 + threadIdx.x;
   if (e >= (long long)gh * gw * quads) return;
@@ -103,6 +106,7 @@ __global__ void __launch_bounds__(256) k_dwc_add(const T* __restrict__ src, cons
 template <typename T>
 __global__ void __launch_bounds__(256) k_dwc_wgrad(const T* __restrict__ V, const T* __restrict__ dO, float* __restrict__ part,
                                                   int n, int d, int prefix, int gh, int gw, int ks, int tpc) {
+  pdl_wait();
   __shared__ float red[256][7][4];
   const int chunk = blockIdx.x, bh = blockIdx.y, a = blockIdx.z, half = ks / 2;
   const int quads = d / 4, lanes = 256 / quads, q = (int)threadIdx.x % quads, tl = (int)threadIdx.x / quads, c = 4 * q;
@@ -151,6 +155,7 @@ __global__ void __launch_bounds__(256) k_dwc_wgrad(const T* __restrict__ V, cons
 template <typename T>
 __global__ void __launch_bounds__(256) k_dwc_wgrad3(const T* __restrict__ V, const T* __restrict__ dO, float* __restrict__ part,
                                                    int n, int d, int prefix, int gh, int gw, int tpc) {
+  pdl_wait();
   __shared__ float red[256][9][4];
   const int chunk = blockIdx.x, bh = blockIdx.y;
   const int quads = d / 4, lanes = 256 / quads, q = (int)threadIdx.x % quads, tl = (int)threadIdx.x / quads, c = 4 * q;
@@ -198,6 +203,7 @@ __global__ void __launch_bounds__(256) k_dwc_wgrad3(const T* __restrict__ V, con
 // grid (ceil(count / 128), H): warp w of a CTA adds the parts w, w + 8, ... for 128 consecutive elements, the eight warps
 // are added in a fixed order.
 __global__ void __launch_bounds__(256) k_dwc_wreduce(const float* __restrict__ part, float* __restrict__ dW, int B, int H, int chunks, int count) {
+  pdl_wait();
   __shared__ float4 red[8][32];
   const int h = blockIdx.y, w = threadIdx.x >> 5, l = threadIdx.x & 31;
   const int e = (blockIdx.x * 32 + l) * 4, P = B * chunks;

@@ -15,6 +15,7 @@ template <int D> __host__ __device__ constexpr size_t exact_smem_bytes() { retur
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_exact_fwd(const T* __restrict__ Q, const T* __restrict__ K, const T* __restrict__ V,
                                                   T* __restrict__ O, int n, float nscale /* -log2(e) / lambda */, int map_mode) {
+  pdl_wait();
   constexpr int P = D + 4, DC = D / 16, GP = 64 + 4;
   extern __shared__ __align__(16) float ex_smem[];
   float* Qs = ex_smem; float* Ks = Qs + 64 * P; float* Vs = Ks + 64 * P; float* Gs = Vs + 64 * P;

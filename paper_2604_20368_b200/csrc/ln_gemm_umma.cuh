@@ -65,6 +65,7 @@ template <int D, bool DWC = false>
 __global__ void __launch_bounds__(256, 3) k_nn_umma(const float* __restrict__ E, int lde, const float* __restrict__ mu,
                                                     const bf16* __restrict__ Yimg, const float* __restrict__ ybar,
                                                     bf16* __restrict__ O, int n, int m, int* dev_status, DwcEpi epi = DwcEpi()) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char gu_smem[];
   bf16* sZ = reinterpret_cast<bf16*>(gu_smem);                 // [2][128 * 64]: hi, lo of the E block (K-major image)
   bf16* sY = sZ + 2 * 128 * GU_KB;                             // [2][64 * D]: hi, lo of the Y block (image, rows = K)
@@ -264,6 +265,7 @@ template <int D>
 __global__ void __launch_bounds__(256, 2) k_ntg_umma(const bf16* __restrict__ U, const bf16* __restrict__ Yimg,
                                                      const float* __restrict__ E, int lde, float* __restrict__ G,
                                                      int n, int m, float inv_lambda, int* dev_status) {
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char gu_smem[];
   bf16* sU = reinterpret_cast<bf16*>(gu_smem);                 // [128 x D] K-major image of the U tile
   bf16* sY = sU + 128 * D;                                     // [2 buffers][2 parts][64 * D]

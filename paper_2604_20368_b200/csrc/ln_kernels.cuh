@@ -69,6 +69,7 @@ __device__ __forceinline__ void l1_fetch8(const void* base, bool f32, long long 
 // SM) where a CTA lives too briefly for two of them to hide each other's loads and epilogues.
 template <int QN>
 __global__ void __launch_bounds__(256, QN == 4 ? 2 : 3) k_l1(const L1Args args) {
+  pdl_wait();
   extern __shared__ __align__(16) float l1_smem[];
   const L1Prob pr = args.p[args.jsplits > 1 ? 0 : blockIdx.z];
   const int LG = blockDim.x, TG = blockDim.y, tj = threadIdx.x, ti = threadIdx.y;
@@ -218,6 +219,7 @@ __global__ void __launch_bounds__(256, QN == 4 ? 2 : 3) k_l1(const L1Args args) 
 // =====================================================================================
 __global__ void __launch_bounds__(256) k_wstat_part(const float* __restrict__ C, int ldc, int n, int m, int rows_per_split,
                                                     double* __restrict__ part /* [BH][splits][m][2] */) {
+  pdl_wait();
   __shared__ double red[4][256][2];
   const int bh = blockIdx.y, split = blockIdx.x, nsplit = gridDim.x;
   const int cq = threadIdx.x & 63, rl = threadIdx.x >> 6, c0 = cq * 4;
@@ -268,6 +270,7 @@ __global__ void __launch_bounds__(256) k_wstat_part(const float* __restrict__ C,
 __global__ void __launch_bounds__(256) k_wstat_final(const double* __restrict__ part, int B, int H, int n, int m, int nsplit,
                                                      float eps, float* __restrict__ s_out /* [H][m] */,
                                                      float* __restrict__ mean_out /* NULL or [H][m] */) {
+  pdl_wait();
   __shared__ double red[8][32][2];
   const int h = blockIdx.y, lane = threadIdx.x & 31, w = threadIdx.x >> 5, l = blockIdx.x * 32 + lane;
   const int terms = B * nsplit;
@@ -319,6 +322,7 @@ __global__ void __launch_bounds__(256) k_wstat_final(const double* __restrict__ 
 __global__ void __launch_bounds__(256) k_whiten_bwd(const float* __restrict__ Y, const float* __restrict__ dYtpart, int nchunks,
                                                     const float* __restrict__ s, const float* __restrict__ cbar, int B, int H,
                                                     int n, int m, int d, float* __restrict__ kap /* [H][m][2] */) {
+  pdl_wait();
   const int h = blockIdx.y, l = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (l >= m) return;
   float acc = 0.f;
@@ -343,6 +347,7 @@ __global__ void __launch_bounds__(256) k_whiten_bwd(const float* __restrict__ Y,
 // paths that materialise G (fp32 storage, 32-dim heads).
 __global__ void __launch_bounds__(256) k_g_whiten_add(float* __restrict__ G, const float* __restrict__ C, const float* __restrict__ kap,
                                                       int H, int n, int m, int ldm, float inv_lambda) {
+  pdl_wait();
   const int bh = blockIdx.y;
   const long long e = (long long)blockIdx.x * 256 + threadIdx.x;
   if (e >= (long long)n * ldm) return;
@@ -356,6 +361,7 @@ __global__ void __launch_bounds__(256) k_g_whiten_add(float* __restrict__ G, con
 
 // storage type -> fp32 copy
 template <typename T> __global__ void k_to_f32(const T* __restrict__ x, float* __restrict__ y, long long count) {
+  pdl_wait();
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < count) y[i] = to_f(x[i]);
 }
@@ -374,6 +380,7 @@ __host__ __device__ inline int bin_hi(int a, int g, int mb) { return (int)(((uns
 // grid (ceil(m / (256 / (d/4))), BH); thread = (landmark, 4 dims)
 template <typename T>
 __global__ void __launch_bounds__(256) k_pool(const T* __restrict__ K, float* __restrict__ L, PoolGeom g) {
+  pdl_wait();
   const int quads = g.d / 4, lpb = 256 / quads;
   const int l = blockIdx.x * lpb + (int)threadIdx.x / quads, bh = blockIdx.y, c = ((int)threadIdx.x % quads) * 4;
   if (l >= g.m || (int)threadIdx.x >= lpb * quads) return;
@@ -404,6 +411,7 @@ __global__ void __launch_bounds__(256) k_pool(const T* __restrict__ K, float* __
 // lanes are added in a fixed order.  With one thread per (landmark, quad) a 28 x 14 bin is a chain of 392 dependent loads.
 template <typename T>
 __global__ void __launch_bounds__(256) k_pool_wide(const T* __restrict__ K, float* __restrict__ L, PoolGeom g) {
+  pdl_wait();
   __shared__ double red[256][4];
   const int quads = g.d / 4, lanes = 256 / quads;
   const int l = blockIdx.x, bh = blockIdx.y, qd = (int)threadIdx.x % quads, tl = (int)threadIdx.x / quads, c = qd * 4;
@@ -439,6 +447,7 @@ constexpr int POOL_EPT = 8;      // elements (of four dims) per thread of k_pool
 template <typename T>
 __global__ void __launch_bounds__(256, 4) k_pool_bwd(const float* __restrict__ dKpart, const float* __restrict__ dL, T* __restrict__ dK,
                                                   PoolGeom g, int pool) {
+  pdl_wait();
   // bin boundaries once per CTA (a division each) instead of several per thread
   __shared__ int rlo[256], rhi[256], clo[256], chi[256];
   __shared__ int s_lm[POOL_EPT * 256 / 8], s_tap[POOL_EPT * 256 / 8];   // per token of this CTA: its landmark and its tap (even bins)
@@ -567,6 +576,7 @@ __device__ __forceinline__ float4 sum_parts4_strided(const float* __restrict__ p
 template <typename TO>
 __global__ void __launch_bounds__(256) k_reduce3_wide(const float* __restrict__ p0, int n0, const float* __restrict__ p1, int n1,
                                                       const float* __restrict__ p2, int n2, TO* __restrict__ out, int count) {
+  pdl_wait();
   __shared__ float4 red[8][32];
   const int bh = blockIdx.y, w = threadIdx.x >> 5, l = threadIdx.x & 31;
   const int e = (blockIdx.x * 32 + l) * 4;
@@ -594,6 +604,7 @@ __global__ void __launch_bounds__(256) k_reduce3_wide(const float* __restrict__ 
 template <typename T>
 __global__ void __launch_bounds__(256) k_filter_grad(const T* __restrict__ X, const float* __restrict__ dL, float* __restrict__ dF,
                                                      PoolGeom g, int B) {
+  pdl_wait();
   __shared__ double red[256][4];
   const int quads = g.d / 4, lanes = 256 / quads;
   const int tap = blockIdx.x, h = blockIdx.y, qd = (int)threadIdx.x % quads, tl = (int)threadIdx.x / quads, c = qd * 4;
@@ -640,6 +651,7 @@ __global__ void __launch_bounds__(256) k_filter_grad(const T* __restrict__ X, co
 }
 // dF[e] = sum over the splits of part[split][e], in order; count = H taps d (a multiple of 4)
 __global__ void __launch_bounds__(256) k_filter_reduce(const float* __restrict__ part, int splits, float* __restrict__ dF, int count) {
+  pdl_wait();
   const int e = (blockIdx.x * 256 + threadIdx.x) * 4;
   if (e >= count) return;
   st4(dF + e, sum_parts4(part, splits, count, e));
@@ -649,6 +661,7 @@ __global__ void __launch_bounds__(256) k_filter_reduce(const float* __restrict__
 template <typename TO>
 __global__ void k_reduce3(const float* __restrict__ p0, int n0, const float* __restrict__ p1, int n1,
                           const float* __restrict__ p2, int n2, TO* __restrict__ out, int count) {
+  pdl_wait();
   const int bh = blockIdx.y;
   const int e = (blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (e >= count) return;
@@ -668,6 +681,7 @@ template <typename TU, int D>
 __global__ void __launch_bounds__(256) k_tn(const float* __restrict__ E, int lde, const float* __restrict__ mu,
                                             const TU* __restrict__ U, float* __restrict__ part,
                                             float* __restrict__ colsum_part, int n, int m, int rpc) {
+  pdl_wait();
   constexpr int DC = D / 16;
   __shared__ __align__(16) float Es[32][64 + 4];
   __shared__ __align__(16) float Us[32][D + 4];
@@ -754,6 +768,7 @@ template <typename TO, int D>
 __global__ void __launch_bounds__(256) k_nn(const float* __restrict__ E, int lde, const float* __restrict__ mu,
                                             const float* __restrict__ Y, const float* __restrict__ ybar,
                                             TO* __restrict__ O, int n, int m) {
+  pdl_wait();
   constexpr int DC = D / 16;
   __shared__ __align__(16) float Es[64][32 + 4];
   __shared__ __align__(16) float Ys[32][D + 4];
@@ -842,6 +857,7 @@ template <typename TU, int D>
 __global__ void __launch_bounds__(256) k_nt_g(const TU* __restrict__ U, const float* __restrict__ Y,
                                               const float* __restrict__ E, int lde, float* __restrict__ G,
                                               int n, int m, float inv_lambda) {
+  pdl_wait();
   constexpr int DK = (D < 64) ? D : 64;
   __shared__ __align__(16) float Us[64][DK + 4];
   __shared__ __align__(16) float Ys[64][DK + 4];
@@ -905,6 +921,7 @@ __global__ void __launch_bounds__(256) k_sign_rows(const TT* __restrict__ tok, c
                                                    const float* __restrict__ G, int ldg, TO* __restrict__ out,
                                                    int n, int m, int lper = 0, const float* __restrict__ Gk = nullptr,
                                                    float gscale = 1.f) {
+  pdl_wait();
   constexpr int DC = D / 16;
   __shared__ __align__(16) float Ls[32][D + 4];
   __shared__ __align__(16) float Gs[64][32 + 4];
@@ -994,6 +1011,7 @@ __global__ void __launch_bounds__(256) k_sign_cols(const TT* __restrict__ tok, c
                                                    const float* __restrict__ G, int ldg, float* __restrict__ part,
                                                    int n, int m, int rpc, const float* __restrict__ Gk = nullptr,
                                                    float gscale = 1.f) {
+  pdl_wait();
   constexpr int DC = D / 16;
   __shared__ __align__(16) float Ts[32][D + 4];
   __shared__ __align__(16) float Gs[32][64 + 4];
@@ -1539,6 +1557,7 @@ template <int CL>
 __global__ void __launch_bounds__(256) k_ns_pinv(int m, int T, float eps, float alpha_in, const float* W,
                                                  float* Wr, float* P, float* Xh, NsHdr* hdr, float* X,
                                                  float* resid) {
+  pdl_wait();
   __shared__ NsSmem sm;
   __shared__ float red[2 * 256 + 8];
   const int b = blockIdx.x / CL, crank = blockIdx.x % CL;
@@ -1571,6 +1590,7 @@ __global__ void __launch_bounds__(256) k_ns_pinv_bwd(int m, int T, float eps, fl
                                                      float* Wr, float* P, float* Hm, float* Ga, float* Gb,
                                                      float* Xh_scratch, const float* Xh_given, NsHdr* hdr,
                                                      const float* dX, float* dW) {
+  pdl_wait();
   __shared__ NsSmem sm;
   __shared__ float red[2 * 256 + 8];
   const int b = blockIdx.x / CL, crank = blockIdx.x % CL;
@@ -1598,6 +1618,7 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
                                                  float* P, float* Xh, float* Ph, NsHdr* hdr, const float* Mpart, int nchunks,
                                                  float* Mout, float* Y, float* Yt, float* ybar, int* dev_status,
                                                  long long hslot, bf16* Yimg, int phase, int solver = 0, float* cgws = nullptr) {
+  pdl_wait();
   // solver: 0 = Newton-Schulz (Alg. 2) and Y = X_T M; 1 = conjugate gradients on (W + eps I) Y = M (Sec. 5.3, Table 4;
   // the single-CTA instantiation without tensor cores only), cgws = 4 m D doubles of scratch per head
   // phase: bit 0 = Newton-Schulz (needs W only), bit 1 = everything that needs M (sum of the partials, Y, map fold).
@@ -1749,6 +1770,7 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
                                                  float* dWm, float* dXm, float* dY, float* dM, float* GW, int* dev_status,
                                                  long long hslot, bf16* dMimg, int sym, int solver = 0, const float* Ysaved = nullptr,
                                                  float* cgws = nullptr, int phase = 3) {
+  pdl_wait();
   // phase: bit 0 = dY, dX and dM (what the key-side kernels wait for), bit 1 = the adjoint of the iteration and GW.
   // The two halves may run as two launches on one stream: the key-side sign pass then starts after the first.
   // solver 1 (conjugate gradients, the fp32 single-CTA instantiation only): the solve is differentiated as the linear
@@ -1874,6 +1896,7 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
 // kernels do (bit 1 of the status word) and returns normally.
 // =====================================================================================
 __global__ void k_selftest_wait(int probes, int* dev_status) {
+  pdl_wait();
   __shared__ __align__(8) unsigned long long mbar;
   if (threadIdx.x == 0) umma::mbar_init(&mbar, 1);
   __syncthreads();
@@ -1896,6 +1919,7 @@ constexpr int kProbeChains = 8;
 // in 3 instructions); 4: mix 2 with scalar and packed instructions in separate runs; 5: mix 2 with scalar instructions
 // only.  Lane-operations per chain and step: 2, 2, 6, 4, 6, 6.
 __global__ void __launch_bounds__(256) k_fp32_add_probe(int iters, int mode, float* sink) {
+  pdl_wait();
   const float x = sink[0];                       // a run-time value the compiler cannot fold
   float a[kProbeChains], b[kProbeChains];
 #pragma unroll

@@ -92,6 +92,7 @@ template <int D>
 __global__ void __launch_bounds__(256, 3) k_tn_mma(const float* __restrict__ E, int lde, const float* __restrict__ mu,
                                                    const bf16* __restrict__ U, float* __restrict__ part,
                                                    float* __restrict__ colsum_part, int n, int m, int rpc) {
+  pdl_wait();
   constexpr int KT = TN_KT, LDE = 64 + 8, LDU = D + 8;
   constexpr int NT = D / 16;        // n8-tiles per warp (half of the dims)
   constexpr int STAGE_BYTES = KT * 64 * 4 + KT * LDU * 2 + KT * 4;
@@ -226,6 +227,7 @@ template <int D>
 __global__ void __launch_bounds__(256) k_nn_mma(const float* __restrict__ E, int lde, const float* __restrict__ mu,
                                                 const float* __restrict__ Y, const float* __restrict__ ybar,
                                                 bf16* __restrict__ O, int n, int m) {
+  pdl_wait();
   constexpr int KL = 32;            // landmarks per step
   constexpr int LDZ = KL + 8, LDY = D + 8;
   constexpr int NT = D / 16;
@@ -317,6 +319,7 @@ template <int D>
 __global__ void __launch_bounds__(256) k_nt_g_mma(const bf16* __restrict__ U, const float* __restrict__ Y,
                                                   const float* __restrict__ E, int lde, float* __restrict__ G,
                                                   int n, int m, float inv_lambda) {
+  pdl_wait();
   constexpr int DK = (D < 64) ? D : 64;
   constexpr int LD = DK + 8;
   __shared__ __align__(16) bf16 Us[64][LD];

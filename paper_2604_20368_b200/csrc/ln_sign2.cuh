@@ -48,6 +48,7 @@ template <typename TT, typename TO, int NR>
 __global__ void __launch_bounds__(256, 2) k_sign2(const TT* __restrict__ tok, const float* __restrict__ Lm,
                                                   const float* __restrict__ G, int ldg, TO* __restrict__ rows,
                                                   float* __restrict__ part, int n, int m, int D, int rpc) {
+  pdl_wait();
   extern __shared__ __align__(16) float s2_smem[];
   const int TG = blockDim.y, tc = threadIdx.x, tt = threadIdx.y;
   const int tid = tt * 16 + tc, nthr = 16 * TG, TT8 = 8 * TG, warp = tid >> 5, lane = tid & 31, nwarps = nthr >> 5;

@@ -47,6 +47,7 @@ static_assert((size_t)(128 * 128 + 2 * GU_KB * 128) * sizeof(bf16) <= sizeof(flo
 
 // Scale and offset of every landmark value (see fold_pair): SB[bh][j][0][c] = s, SB[bh][j][1][c] = b.
 __global__ void __launch_bounds__(256) k_fold_landmarks(const float* __restrict__ Lm, float* __restrict__ SB, int D, long long count) {
+  pdl_wait();
   const long long e = (long long)blockIdx.x * 256 + threadIdx.x;     // index into Lm [BH * m][D]
   if (e >= count) return;
   const long long row = e / D; const int c = (int)(e % D);
@@ -79,6 +80,7 @@ __global__ void __launch_bounds__(256, 2) k_sign3(const bf16* __restrict__ tok, 
                                                   const float* __restrict__ A, int lda, TO* __restrict__ rows,
                                                   float* __restrict__ part, int n, int m, float inv_lambda, int* dev_status,
                                                   const float* __restrict__ kap /* NULL or [H][m][2] */, int H) {
+  pdl_wait();
   extern __shared__ __align__(128) float s3_smem[];
   __shared__ __align__(8) unsigned long long mbar_y, mbar_mma;
   __shared__ uint32_t tmem_base;

@@ -482,6 +482,48 @@ def test_runs_twice_bit_identical():
         assert torch.equal(a[k], b[k]), k
 
 
+@pytest.mark.parametrize("name,B", [("cfg1", 1), ("cfg2", 4), ("cfg5_m256_T4", 1)])
+def test_back_to_back_steps_and_a_captured_step_match(name, B):
+    """The kernels are launched as programmatic dependents of one another.  Steps on alternating inputs that reuse the
+    same buffers without a pause, and the same step replayed from a CUDA graph, give the bits of a step run alone."""
+    cfg = synth.shrink(synth.CONFIGS[name], B=B)
+    inp = synth.make_inputs(cfg)
+    a = [inp[k].to(DEV) for k in ("Q", "K", "V", "dO")]
+    b = [t.flip(0, 2).contiguous() for t in a]
+    p = ln.problem_from_config(cfg, whiten=inp["whiten"].to(DEV))
+    cur = [torch.empty_like(t) for t in a]
+    saved = torch.empty(ln.laplace_nystrom_saved_bytes(p), dtype=torch.uint8, device=DEV)
+    ws = torch.empty(ln.laplace_nystrom_workspace_bytes(p, True), dtype=torch.uint8, device=DEV)
+
+    def step(src):
+        for t, v in zip(cur, src):
+            t.copy_(v)
+        O = ln.laplace_nystrom_fwd(p, *cur[:3], saved=saved, ws=ws)
+        return [O] + list(ln.laplace_nystrom_bwd(p, *cur, saved, ws=ws)[:3])
+
+    ref = []
+    for src in (a, b):
+        ref.append(step(src))
+        torch.cuda.synchronize()
+    got = [step((a, b)[i & 1]) for i in range(20)]
+    torch.cuda.synchronize()
+    for i, g in enumerate(got):
+        assert all(torch.equal(x, y) for x, y in zip(g, ref[i & 1])), i
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        step(a)
+    st.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        out = step(a)
+    for _ in range(3):
+        for t in out:
+            t.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(x, y) for x, y in zip(out, ref[0]))
+
+
 @pytest.mark.parametrize("name,B", [("cfg2", 8), ("cfg3", 2), ("cfg4a", 1), ("cfg5_m128_T8", 1), ("cfg5_m256_T4", 1)])
 def test_overlap_on_the_side_stream_changes_no_bit(name, B):
     """With the per-head kernels on the library's second stream (the default) the results are the bits of
