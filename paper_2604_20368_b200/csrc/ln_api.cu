@@ -557,14 +557,16 @@ int fwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
                                  pl.cg ? 1 : 0, w.cg));
     };
     // conjugate gradients (Sec. 5.3): fp32, one CTA per head, whatever the storage type
+    const size_t mid_smem = TC ? sizeof(MmaGemmSmem) : (m <= 64 && kResFwdSmem > sizeof(GemmSmem) ? kResFwdSmem : sizeof(GemmSmem));
     if (pl.cg) { launch(k_mid_fwd<D, false, 0>, sizeof(NsSmem)); return; }
-    // general (non-symmetric) matrix: the mma.sync or FFMA engine, shared by the CTAs of a cluster beyond 64 landmarks
-    if (two && m > 64) launch(k_mid_fwd<D, TC, 0, kMidCluster>, sizeof(NsSmem), kMidCluster);
-    else if (two) launch(k_mid_fwd<D, TC, 0>, sizeof(NsSmem));
+    // two landmark sets (general matrix) or fp32 storage: the mma.sync or FFMA engine, shared by the CTAs of a cluster
+    // beyond 64 landmarks
+    if ((two || !TC) && m > 64) launch(k_mid_fwd<D, TC, 0, kMidCluster>, mid_smem, kMidCluster);
+    else if (two) launch(k_mid_fwd<D, TC, 0>, mid_smem);
     else if (TC && m <= 64) launch(k_mid_fwd<D, TC, TC ? 64 : 0>, 3 * kUmmaMatBytes64);
     else if (TC && m <= 128) launch(k_mid_fwd<D, TC, TC ? 128 : 0>, 3 * kUmmaMatBytes);
     else if (TC) launch(k_mid_fwd<D, TC, TC ? 256 : 0, TC ? kU2Cluster : 1>, 3 * kUmmaMatBytes, kU2Cluster);   // m > 128: a cluster per head
-    else launch(k_mid_fwd<D, TC, 0>, sizeof(NsSmem));
+    else launch(k_mid_fwd<D, TC, 0>, mid_smem);
   };
   {
     L1Args a;
@@ -718,13 +720,14 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
                                                  umma_prod ? reinterpret_cast<bf16*>(w.dMimg) : nullptr, two ? 0 : 1,
                                                  pl.cg ? 1 : 0, x.Y, w.cg, phase));
     };
+    const size_t mid_smem = TC ? sizeof(MmaGemmSmem) : (m <= 64 ? kResBwdSmem : sizeof(GemmSmem));
     if (pl.cg) { launch(k_mid_bwd<D, false, 0>, sizeof(NsSmem)); return; }
-    if (two && m > 64) launch(k_mid_bwd<D, TC, 0, kMidCluster>, sizeof(NsSmem), kMidCluster);
-    else if (two) launch(k_mid_bwd<D, TC, 0>, sizeof(NsSmem));
+    if ((two || !TC) && m > 64) launch(k_mid_bwd<D, TC, 0, kMidCluster>, mid_smem, kMidCluster);
+    else if (two) launch(k_mid_bwd<D, TC, 0>, mid_smem);
     else if (TC && m <= 64) launch(k_mid_bwd<D, TC, TC ? 64 : 0>, 4 * kUmmaMatBytes64);
     else if (TC && m <= 128) launch(k_mid_bwd<D, TC, TC ? 128 : 0>, 3 * kUmmaMatBytes);
     else if (TC) launch(k_mid_bwd<D, TC, TC ? 256 : 0, TC ? kU2Cluster : 1>, 3 * kUmmaMatBytes, kU2Cluster);
-    else launch(k_mid_bwd<D, TC, 0>, sizeof(NsSmem));
+    else launch(k_mid_bwd<D, TC, 0>, mid_smem);
   };
   // key-side products: g^R = (V dM^T) o R^T / lambda and dV = R^T dM (they need dM from the per-head kernel)
   auto launch_ntg_R = [&](cudaStream_t s) {
@@ -920,16 +923,18 @@ NsWs carve_ns_ws(int batch, int m, int T, void* base) {
   return w;
 }
 
-// CTAs of a thread-block cluster that share one matrix of the stand-alone Newton-Schulz entry points (64 x 64 output
-// tiles of every product are dealt out to them)
-int ns_cluster(int m) { return m > 128 ? 8 : (m > 64 ? 4 : 1); }
+// CTAs of a thread-block cluster that share one matrix of the stand-alone Newton-Schulz entry points (the output tiles of
+// every product are dealt out to them); up to 64 the matrices of a step fit one CTA's shared memory
+int ns_cluster(int m) { return m > 64 ? 8 : 1; }
 void launch_ns_pinv(int batch, int m, int iters, float eps, float alpha, const float* W, const NsWs& w, float* Xh, float* X,
                     float* resid, cudaStream_t st) {
   const int cl = ns_cluster(m);
   auto go = [&](auto kern) {
-    LN_LAUNCH("k_ns_pinv", st, launch_clustered(kern, batch * cl, cl, 0, st, m, iters, eps, alpha, W, w.Wr, w.P, Xh, w.hdr, X, resid));
+    const size_t smem = cl == 1 ? kResFwdSmem : sizeof(GemmSmem);
+    want_smem(kern, smem);
+    LN_LAUNCH("k_ns_pinv", st, launch_clustered(kern, batch * cl, cl, smem, st, m, iters, eps, alpha, W, w.Wr, w.P, Xh, w.hdr, X, resid));
   };
-  if (cl == 8) go(k_ns_pinv<8>); else if (cl == 4) go(k_ns_pinv<4>); else go(k_ns_pinv<1>);
+  if (cl == 8) go(k_ns_pinv<8>); else go(k_ns_pinv<1>);
 }
 }  // namespace
 
@@ -1243,10 +1248,12 @@ int ns_pinv_bwd(int32_t batch, int32_t m, const float* W, int32_t iters, float r
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int cl = ns_cluster(m);
     auto go = [&](auto kern) {
-      LN_LAUNCH("k_ns_pinv_bwd", st, launch_clustered(kern, batch * cl, cl, 0, st, m, iters, ridge_eps, alpha, W, w.Wr, w.P, w.Hm, w.Ga, w.Gb, w.Xh,
+      const size_t smem = cl == 1 ? kResBwdSmem : sizeof(GemmSmem);
+      want_smem(kern, smem);
+      LN_LAUNCH("k_ns_pinv_bwd", st, launch_clustered(kern, batch * cl, cl, smem, st, m, iters, ridge_eps, alpha, W, w.Wr, w.P, w.Hm, w.Ga, w.Gb, w.Xh,
                                                       X_hist, w.hdr, dX, dW));
     };
-    if (cl == 8) go(k_ns_pinv_bwd<8>); else if (cl == 4) go(k_ns_pinv_bwd<4>); else go(k_ns_pinv_bwd<1>);
+    if (cl == 8) go(k_ns_pinv_bwd<8>); else go(k_ns_pinv_bwd<1>);
   }
   return launch_ok();
 }

@@ -88,13 +88,20 @@ __device__ __forceinline__ void fold_pair(float y, float& s, float& b) {
 // matrix equal in exact arithmetic; without the window the rounding of the sums would pick the winner (Alg. 2's
 // scale depends on the 1- and infinity-norm; any of the tied columns gives a valid subgradient).
 constexpr float kNormTie = 1.f / 16384.f;
+// One warp, the same result in every lane.
 __device__ __forceinline__ void norm_argmax(const float* s, int m, float& mx, int& idx) {
+  const int lane = threadIdx.x & 31;
   mx = -1.f;
-  for (int t = 0; t < m; ++t) mx = fmaxf(mx, s[t]);
+  for (int t = lane; t < m; t += 32) mx = fmaxf(mx, s[t]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   const float thr = mx * (1.f - kNormTie);
-  idx = 0;
-  for (int t = 0; t < m; ++t)
-    if (s[t] >= thr) { idx = t; break; }
+  int first = m;                                    // this lane's lowest index inside the window
+  for (int t = lane; t < m; t += 32)
+    if (s[t] >= thr) { first = t; break; }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) first = min(first, __shfl_xor_sync(0xffffffffu, first, o));
+  idx = first < m ? first : 0;                      // no entry compares (NaN): index 0
 }
 
 // Packed pair arithmetic (two fp32 lanes per instruction): the FP32 pipe does not get faster, but a
@@ -184,6 +191,22 @@ template <int CL> __device__ __forceinline__ void phase_sync() {
   } else {
     __syncthreads();
   }
+}
+
+// Sum of one value per CTA of a cluster, added in rank order; the same result in every thread.  `slots`: CL floats of
+// shared memory that nothing else uses between the last cluster barrier before the call and the one inside it.
+template <int CL> __device__ __forceinline__ float cluster_sum(float v, float* slots, int crank) {
+  if (threadIdx.x < CL) {
+    uint32_t remote;
+    const uint32_t mine = (uint32_t)__cvta_generic_to_shared(slots + crank);
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(mine), "r"((int)threadIdx.x));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
+  }
+  phase_sync<CL>();
+  float s = 0.f;
+#pragma unroll
+  for (int c = 0; c < CL; ++c) s += slots[c];
+  return s;
 }
 
 // Depth-wise convolution branch of the attention block (Eq. 7: Attention = Z V + DWC(V)) as an addition to the output of a

@@ -1087,73 +1087,207 @@ __global__ void __launch_bounds__(256) k_sign_cols(const TT* __restrict__ tok, c
 
 // =====================================================================================
 // Whole-CTA fp32 GEMM on global (L2-resident) row-major matrices:
-//   C = beta * Cin + alpha * op(A) op(B),  op(A) is M x K, op(B) is K x N.
+//   C = beta * Cin + alpha * (op(A) op(B) [+ sgn2 * op2(A2) op2(B2)]) + diag * I,   op(A) is M x K, op(B) is K x N.
 // Executed by all 256 threads of a CTA; ends with __syncthreads(), so a following call may
 // read C.  Cin may equal C (each element is read and written by the same thread).
+//
+// A product of the iteration is a chain link: what it waits for (operands from L2, barriers) counts as much as its
+// multiply-adds.  So a tile stages its operands for up to 128 values of k at once, all copies asynchronous and in
+// flight together (two groups, the second arrives beside the products of the first), instead of 16 values per
+// load - barrier - multiply round; and the k range is dealt out to four groups of 64 threads with 8 x 8 (8 x 4) outputs
+// each, which reads 1 (1.5) shared-memory floats per 4 multiply-adds where 4 x 4 outputs read 2.  The four partial sums
+// meet in shared memory and are added in a fixed order.  Sixteen 128 x 128 matrices, T = 8, eight CTAs each: forward
+// 176 -> 131 us, adjoint 425 -> 273 us (four CTAs and 16-value rounds before).
 // =====================================================================================
-struct GemmSmem { float As[16][64 + 4]; float Bs[16][64 + 4]; };
+constexpr int FG_K = 128;          // values of k staged at a time
+constexpr int FG_KP = FG_K + 4;    // pitch of an operand staged with k along its rows
+constexpr int FG_IP = 64 + 8;      // pitch of an operand staged with k down its columns
+constexpr int FG_RP = 64 + 2;      // pitch of the partial sums
+constexpr int FG_OP = FG_K * FG_IP > 64 * FG_KP ? FG_K * FG_IP : 64 * FG_KP;      // floats of one staged operand
+struct __align__(16) GemmSmem { float op[2][FG_OP]; };
+static_assert(4 * 64 * FG_RP <= 2 * FG_OP, "the partial sums fit in the operand buffers");
 
-template <bool TRA, bool TRB>
-__device__ void cta_gemm(int M, int N, int K, const float* A, int lda, const float* Bm, int ldb,
-                         float* C, int ldc, float alpha, float beta, const float* Cin, GemmSmem& sm, int part = 0, int nparts = 1) {
-  // nparts CTAs of a cluster share the product: output tile t goes to CTA t % nparts
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  int tile = 0;
-  for (int i0 = 0; i0 < M; i0 += 64)
-    for (int j0 = 0; j0 < N; j0 += 64) {
-      if ((tile++) % nparts != part) continue;
-      float acc[4][4];
+__device__ __forceinline__ void fg_copy4(float* dst, const float* src, bool in) {      // 4 bytes, zero where !in
+  const int sz = in ? 4 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(umma::s32(dst)), "l"(src), "r"(sz) : "memory");
+}
+__device__ __forceinline__ void fg_copy16(float* dst, const float* src, bool in) {
+  const int sz = in ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(umma::s32(dst)), "l"(src), "r"(sz) : "memory");
+}
+// rows [r0, r1) and columns [c0, c1), c1 - c0 <= W, of a block: src[r * ld + c] to dst[r * pitch + c]; zero from row nr and
+// column ncv on.  A thread keeps its column, so an element costs a predicate, two additions and the copy.
+template <int W>
+__device__ __forceinline__ void fg_stage(float* dst, int pitch, const float* src, int ld, int r0, int r1, int c0, int c1, int nr, int ncv) {
+  if (((ld | ncv | c0) & 3) == 0 && (reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+    constexpr int Q = W / 4, RS = 256 / Q;                       // pieces of 16 bytes per row, rows per pass of the CTA
+    const int c = c0 + 4 * (int)(threadIdx.x % Q);
+    int r = r0 + (int)(threadIdx.x / Q);
+    if (c < c1) {
+      const bool cin = c < ncv;
+      const float* p = src + (cin ? r * ld + c : 0);
+      float* q = dst + r * pitch + c;
+#pragma unroll 4
+      for (; r < r1; r += RS) {
+        const bool in = cin && r < nr;
+        fg_copy16(q, in ? p : src, in);
+        p += cin ? RS * ld : 0; q += RS * pitch;
+      }
+    }
+  } else {
+    constexpr int RS = 256 / W;
+    const int c = c0 + (int)(threadIdx.x % W);
+    int r = r0 + (int)(threadIdx.x / W);
+    if (c < c1) {
+      const bool cin = c < ncv;
+      const float* p = src + (cin ? r * ld + c : 0);
+      float* q = dst + r * pitch + c;
+#pragma unroll 4
+      for (; r < r1; r += RS) {
+        const bool in = cin && r < nr;
+        fg_copy4(q, in ? p : src, in);
+        p += cin ? RS * ld : 0; q += RS * pitch;
+      }
+    }
+  }
+}
+// acc[r][s] += sgn * op(A) op(B) for this thread's rows {4 ty + r, 32 + 4 ty + r} and columns {tx + 8 s} of the tile at
+// (i0, j0) and its group's share of k (blocks of four, dealt out in turn)
+template <bool TRA, bool TRB, int TN, bool NEG>
+__device__ __forceinline__ void fg_accumulate(float (&acc)[8][TN / 8], int M, int N, int K, const float* A, int lda, const float* Bm, int ldb,
+                                              int i0, int j0, GemmSmem& sm) {
+  constexpr int NS = TN / 8;
+  const int tid = threadIdx.x, kg = tid >> 6, ty = (tid >> 3) & 7, tx = tid & 7;
+  float* const sA = sm.op[0];
+  float* const sB = sm.op[1];
+  for (int k0 = 0; k0 < K; k0 += FG_K) {
+    const int kc = min(FG_K, K - k0), k4 = (kc + 3) & ~3;
+    const int half = k4 > 32 ? ((k4 / 2 + 15) & ~15) : k4;     // a whole number of four-blocks for every group
+    __syncthreads();                                             // the buffers are free
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      const int ka = h ? half : 0, kb = h ? k4 : half;
+      if (kb > ka) {
+        if (TRA) fg_stage<64>(sA, FG_IP, A + (long long)k0 * lda + i0, lda, ka, kb, 0, 64, kc, M - i0);
+        else     fg_stage<64>(sA, FG_KP, A + (long long)i0 * lda + k0, lda, 0, 64, ka, kb, M - i0, kc);
+        if (TRB) fg_stage<64>(sB, FG_KP, Bm + (long long)j0 * ldb + k0, ldb, 0, TN, ka, kb, N - j0, kc);
+        else     fg_stage<TN>(sB, FG_IP, Bm + (long long)k0 * ldb + j0, ldb, ka, kb, 0, TN, kc, N - j0);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      if (h == 0) asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncthreads();
+      const int ka = h ? half : 0, kb = h ? k4 : half;
+#pragma unroll 1
+      for (int kk = ka + 4 * kg; kk < kb; kk += 16) {
+        float a[8][4];                                          // [row][k]
+        if (TRA) {
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int s = 0; s < 4; ++s) acc[r][s] = 0.f;
-      for (int k0 = 0; k0 < K; k0 += 16) {
-        __syncthreads();
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int idx = tid + e * 256;   // 1024 elements per operand tile
-          if (TRA) {                       // op(A)(i,k) = A[k][i]: i fastest
-            const int kk = idx >> 6, i = idx & 63;
-            sm.As[kk][i] = (k0 + kk < K && i0 + i < M) ? A[(long long)(k0 + kk) * lda + i0 + i] : 0.f;
-          } else {                         // op(A)(i,k) = A[i][k]: k fastest
-            const int i = idx >> 4, kk = idx & 15;
-            sm.As[kk][i] = (k0 + kk < K && i0 + i < M) ? A[(long long)(i0 + i) * lda + k0 + kk] : 0.f;
+          for (int u = 0; u < 4; ++u) {
+            const float4 lo = *reinterpret_cast<const float4*>(sA + (kk + u) * FG_IP + 4 * ty);
+            const float4 hi = *reinterpret_cast<const float4*>(sA + (kk + u) * FG_IP + 32 + 4 * ty);
+            a[0][u] = lo.x; a[1][u] = lo.y; a[2][u] = lo.z; a[3][u] = lo.w;
+            a[4][u] = hi.x; a[5][u] = hi.y; a[6][u] = hi.z; a[7][u] = hi.w;
           }
-          if (TRB) {                       // op(B)(k,j) = B[j][k]: k fastest
-            const int j = idx >> 4, kk = idx & 15;
-            sm.Bs[kk][j] = (k0 + kk < K && j0 + j < N) ? Bm[(long long)(j0 + j) * ldb + k0 + kk] : 0.f;
-          } else {                         // op(B)(k,j) = B[k][j]: j fastest
-            const int kk = idx >> 6, j = idx & 63;
-            sm.Bs[kk][j] = (k0 + kk < K && j0 + j < N) ? Bm[(long long)(k0 + kk) * ldb + j0 + j] : 0.f;
+        } else {
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            const float4 v = *reinterpret_cast<const float4*>(sA + ((r >> 2) * 32 + 4 * ty + (r & 3)) * FG_KP + kk);
+            a[r][0] = v.x; a[r][1] = v.y; a[r][2] = v.z; a[r][3] = v.w;
           }
         }
-        __syncthreads();
+        if (NEG) {
 #pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-          const float4 a = *reinterpret_cast<const float4*>(&sm.As[kk][ty * 4]);
-          const float4 b = *reinterpret_cast<const float4*>(&sm.Bs[kk][tx * 4]);
-          const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+          for (int r = 0; r < 8; ++r)
 #pragma unroll
-          for (int r = 0; r < 4; ++r)
+            for (int u = 0; u < 4; ++u) a[r][u] = -a[r][u];
+        }
 #pragma unroll
-            for (int s = 0; s < 4; ++s) acc[r][s] = fmaf(av[r], bv[s], acc[r][s]);
+        for (int q = 0; q < NS; ++q) {
+          float b[4];
+          if (TRB) {
+            const float4 v = *reinterpret_cast<const float4*>(sB + (tx + 8 * q) * FG_KP + kk);
+            b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
+          } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) b[u] = sB[(kk + u) * FG_IP + tx + 8 * q];
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int r = 0; r < 8; ++r) acc[r][q] = fmaf(a[r][u], b[u], acc[r][q]);
         }
       }
+    }
+  }
+}
+
+// the second product of a call: op2(A2) op2(B2), added (sgn > 0) or subtracted; A2 == NULL: none
+struct FgSecond { const float* A; int lda; const float* B; int ldb; int K; };
+
+template <bool TRA, bool TRB, int TN, bool TWO, bool TRA2, bool TRB2, bool NEG2>
+__device__ void cta_gemm_tiles(int M, int N, int K, const float* A, int lda, const float* Bm, int ldb, float* C, int ldc, float alpha,
+                               float beta, const float* Cin, float diag, const FgSecond& sec, GemmSmem& sm, int part, int nparts) {
+  // nparts CTAs of a cluster share the product: output tile t goes to CTA t % nparts
+  constexpr int NS = TN / 8;
+  const int tid = threadIdx.x, kg = tid >> 6, ty = (tid >> 3) & 7, tx = tid & 7;
+  int tile = 0;
+  for (int i0 = 0; i0 < M; i0 += 64)
+    for (int j0 = 0; j0 < N; j0 += TN) {
+      if ((tile++) % nparts != part) continue;
+      float acc[8][NS];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int i = i0 + ty * 4 + r;
-        if (i >= M) continue;
+      for (int r = 0; r < 8; ++r)
 #pragma unroll
-        for (int s = 0; s < 4; ++s) {
-          const int j = j0 + tx * 4 + s;
-          if (j >= N) continue;
-          float v = alpha * acc[r][s];
-          if (beta != 0.f) v += beta * Cin[(long long)i * ldc + j];
-          C[(long long)i * ldc + j] = v;
+        for (int s = 0; s < NS; ++s) acc[r][s] = 0.f;
+      fg_accumulate<TRA, TRB, TN, false>(acc, M, N, K, A, lda, Bm, ldb, i0, j0, sm);
+      if constexpr (TWO) fg_accumulate<TRA2, TRB2, TN, NEG2>(acc, M, N, sec.K, sec.A, sec.lda, sec.B, sec.ldb, i0, j0, sm);
+      __syncthreads();                                           // the operands have been read
+      float* const R = sm.op[0];
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int s = 0; s < NS; ++s) R[(kg * 64 + (r >> 2) * 32 + 4 * ty + (r & 3)) * FG_RP + tx + 8 * s] = acc[r][s];
+      __syncthreads();
+      constexpr int RS = 256 / TN, NE = 64 / RS;                // a thread adds up NE elements of one column
+      const int c = tid % TN, j = j0 + c, r0 = tid / TN;
+      if (j < N) {
+        const int nr = M - i0, at = (i0 + r0) * ldc + j;
+#pragma unroll
+        for (int h = 0; h < NE; h += 8) {
+          float ci[8], v[8];
+          if (beta != 0.f) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) ci[u] = r0 + (h + u) * RS < nr ? Cin[at + (h + u) * RS * ldc] : 0.f;
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const float* q = R + (r0 + (h + u) * RS) * FG_RP + c;
+            v[u] = alpha * ((q[0] + q[64 * FG_RP]) + (q[128 * FG_RP] + q[192 * FG_RP]));
+          }
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int r = r0 + (h + u) * RS;
+            if (beta != 0.f) v[u] += beta * ci[u];
+            if (i0 + r == j) v[u] += diag;
+            if (r < nr) C[at + (h + u) * RS * ldc] = v[u];
+          }
         }
       }
     }
   __syncthreads();
+}
+
+// Tile width: 64 columns, or 32 where the narrower tiles fill the CTAs of the cluster better (a tile costs about 4 : 3).
+template <bool TRA, bool TRB, bool TWO = false, bool TRA2 = false, bool TRB2 = false, bool NEG2 = false>
+__device__ __forceinline__ void cta_gemm(int M, int N, int K, const float* A, int lda, const float* Bm, int ldb, float* C, int ldc, float alpha,
+                                         float beta, const float* Cin, float diag, GemmSmem& sm, int part, int nparts, FgSecond sec = {}) {
+  const int ti = (M + 63) / 64, r64 = (ti * ((N + 63) / 64) + nparts - 1) / nparts, r32 = (ti * ((N + 31) / 32) + nparts - 1) / nparts;
+  if (4 * r64 <= 3 * r32) cta_gemm_tiles<TRA, TRB, 64, TWO, TRA2, TRB2, NEG2>(M, N, K, A, lda, Bm, ldb, C, ldc, alpha, beta, Cin, diag, sec, sm, part, nparts);
+  else cta_gemm_tiles<TRA, TRB, 32, TWO, TRA2, TRB2, NEG2>(M, N, K, A, lda, Bm, ldb, C, ldc, alpha, beta, Cin, diag, sec, sm, part, nparts);
 }
 
 // Shared memory of the per-head kernels: one of the two GEMM engines is used per instantiation.
@@ -1168,15 +1302,233 @@ __device__ __forceinline__ void ns_gemm(int M, int N, int K, const float* A, int
   if (TC) {
     cta_gemm_mma<TRA, TRB>(M, N, K, A, lda, Bm, ldb, C, ldc, alpha, beta, Cin, diag, sm.t, part, nparts);
   } else {
-    // the diagonal term is folded into the product by the CTA that owns the tile: added after its own tiles are stored
-    cta_gemm<TRA, TRB>(M, N, K, A, lda, Bm, ldb, C, ldc, alpha, beta, Cin, sm.f, part, nparts);
-    if (diag != 0.f) {
-      const int lim = M < N ? M : N, tiles_n = (N + 63) / 64;
-      for (int i = threadIdx.x; i < lim; i += 256)
-        if (((i / 64) * tiles_n + i / 64) % nparts == part) C[(long long)i * ldc + i] += diag;
-      __syncthreads();
+    cta_gemm<TRA, TRB>(M, N, K, A, lda, Bm, ldb, C, ldc, alpha, beta, Cin, diag, sm.f, part, nparts);
+  }
+}
+
+// =====================================================================================
+// fp32 Newton-Schulz and its adjoint for m <= 64 by one CTA, every matrix of a step resident in shared memory (row-major,
+// pitch 68: all four transpose variants of a product read it without bank conflicts).  A product is then no longer a
+// round trip through L2: thread (ty, tx) of one of four groups of 64 threads forms rows ty + 8 r, columns tx + 8 q
+// (r, q < NR = 4, 7 or 8, whichever hugs m) over its quarter of k, and the four partial sums are added in a fixed order.
+// At m = 49, T = 6, 32 heads: k_mid_fwd / k_mid_bwd 72 / 141 -> 50 / 93 us (2.2 us a product instead of 4.0).
+// =====================================================================================
+constexpr int RS_P = 68;                          // pitch of a resident matrix
+constexpr int RS_MAT = 64 * RS_P;                 // floats of one
+constexpr int RS_RP = 72;                         // pitch of the partial sums: two buffers of 64 rows
+constexpr size_t rs_smem_bytes(int mats) { return sizeof(float) * ((size_t)mats * RS_MAT + 2 * 64 * RS_RP); }
+constexpr size_t kResFwdSmem = rs_smem_bytes(3), kResBwdSmem = rs_smem_bytes(5);
+
+// acc (+ or -)= op(A) op(B) over this group's share of k (blocks of four, dealt out in turn)
+template <bool TRA, bool TRB, int NR, bool NEG = false>
+__device__ __forceinline__ void rs_mac(float (&acc)[NR][NR], const float* A, const float* Bm, int m) {
+  const int tid = threadIdx.x, kg = tid >> 6, ty = (tid >> 3) & 7, tx = tid & 7;
+#pragma unroll 1
+  for (int kk = 4 * kg; kk < m; kk += 16) {
+    float a[NR][4];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (TRA) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[r][u] = A[(kk + u) * RS_P + ty + 8 * r];
+      } else {
+        const float4 v = *reinterpret_cast<const float4*>(A + (ty + 8 * r) * RS_P + kk);
+        a[r][0] = v.x; a[r][1] = v.y; a[r][2] = v.z; a[r][3] = v.w;
+      }
+      if (NEG) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[r][u] = -a[r][u];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < NR; ++q) {
+      float b[4];
+      if (TRB) {
+        const float4 v = *reinterpret_cast<const float4*>(Bm + (tx + 8 * q) * RS_P + kk);
+        b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
+      } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) b[u] = Bm[(kk + u) * RS_P + tx + 8 * q];
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int r = 0; r < NR; ++r) acc[r][q] = fmaf(a[r][u], b[u], acc[r][q]);
     }
   }
+}
+template <int NR> __device__ __forceinline__ void rs_zero(float (&acc)[NR][NR]) {
+#pragma unroll
+  for (int r = 0; r < NR; ++r)
+#pragma unroll
+    for (int q = 0; q < NR; ++q) acc[r][q] = 0.f;
+}
+// The sum over the four groups: v[u] = element (row tid / 64 + 4 u, column tid % 64), zero outside m x m.  Every operand of
+// the product has been read when this returns.
+template <int NR>
+__device__ __forceinline__ void rs_sum(const float (&acc)[NR][NR], float* R, int m, float (&v)[2 * NR]) {
+  const int tid = threadIdx.x, kg = tid >> 6, ty = (tid >> 3) & 7, tx = tid & 7;
+  float* const mine = R + (kg & 1) * (64 * RS_RP) + ty * RS_RP + tx;
+  if (kg < 2) {
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+#pragma unroll
+      for (int q = 0; q < NR; ++q) mine[8 * r * RS_RP + 8 * q] = acc[r][q];
+  }
+  __syncthreads();
+  if (kg >= 2) {
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+#pragma unroll
+      for (int q = 0; q < NR; ++q) mine[8 * r * RS_RP + 8 * q] += acc[r][q];
+  }
+  __syncthreads();
+  const int c = tid & 63, r0 = tid >> 6;
+#pragma unroll
+  for (int u = 0; u < 2 * NR; ++u) {
+    const float* q = R + (r0 + 4 * u) * RS_RP + c;
+    v[u] = (c < m && r0 + 4 * u < m) ? q[0] + q[64 * RS_RP] : 0.f;
+  }
+}
+// this thread's elements -> a resident matrix (padding included) and, where dst != NULL, an [m][m] matrix in global memory
+template <int NE>
+__device__ __forceinline__ void rs_put(const float (&v)[NE], float* mat, float* dst, int m) {
+  const int c = threadIdx.x & 63, r0 = threadIdx.x >> 6;
+#pragma unroll
+  for (int u = 0; u < NE; ++u) {
+    const int r = r0 + 4 * u;
+    if (mat) mat[r * RS_P + c] = v[u];
+    if (dst && r < m && c < m) dst[r * m + c] = v[u];
+  }
+}
+
+// One [m][m] matrix from global memory into a resident one, asynchronously (rows and columns >= m are left alone).
+__device__ __forceinline__ void rs_load_async(float* mat, const float* src, int m) {
+  const int c = threadIdx.x & 63;
+  if (c < m)
+    for (int r = threadIdx.x >> 6; r < m; r += 4) fg_copy4(mat + r * RS_P + c, src + r * m + c, true);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+template <int NR>
+__device__ void ns_forward_res(int m, int T, float eps, float alpha_in, const float* W, float* Wr, float* Xh, NsHdr* hdr, float* smem,
+                               float* red, float* Qh) {
+  constexpr int NE = 2 * NR;
+  const int tid = threadIdx.x, c = tid & 63, r0 = tid >> 6, mm = m * m;
+  float* sW = smem; float* sX = smem + RS_MAT; float* sQ = smem + 2 * RS_MAT; float* R = smem + 3 * RS_MAT;
+  float v[NE];
+#pragma unroll
+  for (int u = 0; u < NE; ++u) {
+    const int r = r0 + 4 * u;
+    v[u] = (r < m && c < m) ? W[r * m + c] + (r == c ? eps : 0.f) : 0.f;
+  }
+  rs_put(v, sW, Wr, m);
+  __syncthreads();
+  if (tid < 128) {                                 // column sums, row sums (rotated start: no bank conflicts)
+    const bool cols = tid < 64;
+    float t = 0.f;
+    if (c < 8 * NR)
+#pragma unroll 8
+      for (int i = 0; i < m; ++i) {
+        int j = i + c; j = j >= m ? j - m : j;
+        if (j >= m) j = 0;                         // c >= m: the sum is not used
+        t += fabsf(cols ? sW[i * RS_P + c] : sW[c * RS_P + j]);
+      }
+    if (c < m) (cols ? red : red + 256)[c] = t;
+  }
+  __syncthreads();
+  if (tid < 64) {                                  // near-ties (duplicated landmarks): the lowest index
+    const bool cols = tid < 32;
+    float mx; int idx;
+    norm_argmax(cols ? red : red + 256, m, mx, idx);
+    if ((tid & 31) == 0) {
+      red[512 + (cols ? 0 : 1)] = mx;
+      if (cols) { hdr->n1 = mx; hdr->jstar = idx; } else { hdr->ninf = mx; hdr->istar = idx; }
+    }
+  }
+  __syncthreads();
+  const float alpha = (alpha_in > 0.f) ? alpha_in : 1.f / (red[512] * red[513]);
+  if (tid == 0) { hdr->auto_alpha = !(alpha_in > 0.f); hdr->alpha = alpha; hdr->pad0 = hdr->pad1 = 0; }
+#pragma unroll
+  for (int u = 0; u < NE; ++u) v[u] = alpha * sW[c < 8 * NR ? c * RS_P + r0 + 4 * u : 0];
+  rs_put(v, sX, Xh, m);
+  __syncthreads();
+  for (int k = 0; k < T; ++k) {
+    float acc[NR][NR];
+    rs_zero(acc);
+    rs_mac<false, false>(acc, sW, sX, m);
+    rs_sum(acc, R, m, v);
+#pragma unroll
+    for (int u = 0; u < NE; ++u) v[u] = ((r0 + 4 * u == c && c < m) ? 2.f : 0.f) - v[u];        // Q_k = 2I - W X_k
+    rs_put(v, sQ, Qh ? Qh + (long long)k * mm : nullptr, m);
+    __syncthreads();
+    rs_zero(acc);
+    rs_mac<false, false>(acc, sX, sQ, m);
+    rs_sum(acc, R, m, v);
+    rs_put(v, sX, Xh + (long long)(k + 1) * mm, m);                                             // X_{k+1} = X_k Q_k
+    __syncthreads();
+  }
+}
+
+// Leaves dLoss/dX_0 in Gout and the part of dW accumulated over the steps in dW (both [m][m], global).
+template <int NR>
+__device__ void ns_backward_res(int m, int T, const float* Wr, const float* Xh, const float* G0, float* dW, float* Gout, float* smem, const float* Qh) {
+  constexpr int NE = 2 * NR;
+  const int tid = threadIdx.x, c = tid & 63, r0 = tid >> 6, mm = m * m;
+  float* sW = smem; float* sA = smem + RS_MAT; float* sQ = smem + 2 * RS_MAT; float* sG = smem + 3 * RS_MAT; float* sH = smem + 4 * RS_MAT;
+  float* R = smem + 5 * RS_MAT;
+  __syncthreads();
+  for (int e = tid; e < 3 * RS_MAT; e += 256) smem[e] = 0.f;       // the padding of the matrices that are copied in
+  float g[NE], dw[NE], v[NE];
+#pragma unroll
+  for (int u = 0; u < NE; ++u) {
+    const int r = r0 + 4 * u;
+    g[u] = (r < m && c < m) ? G0[r * m + c] : 0.f;
+    dw[u] = 0.f;
+  }
+  rs_put(g, sG, nullptr, m);
+  __syncthreads();
+  rs_load_async(sW, Wr, m);
+  if (T > 0) rs_load_async(sA, Xh + (long long)(T - 1) * mm, m);
+  if (T > 0 && Qh) rs_load_async(sQ, Qh + (long long)(T - 1) * mm, m);
+  for (int k = T - 1; k >= 0; --k) {
+    float acc[NR][NR];
+    if (Qh) asm volatile("cp.async.wait_group 1;" ::: "memory");   // A = X_k is here; Q_k may still be on its way
+    else asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (!Qh) {                                                     // Q_k = 2I - Wr X_k once more
+      rs_zero(acc);
+      rs_mac<false, false>(acc, sW, sA, m);
+      rs_sum(acc, R, m, v);
+#pragma unroll
+      for (int u = 0; u < NE; ++u) v[u] = ((r0 + 4 * u == c && c < m) ? 2.f : 0.f) - v[u];
+      rs_put(v, sQ, nullptr, m);
+      __syncthreads();                                             // the partial sums have been read
+    }
+    rs_zero(acc);
+    rs_mac<true, false>(acc, sA, sG, m);                           // H = A^T G
+    rs_sum(acc, R, m, v);
+    rs_put(v, sH, nullptr, m);
+    __syncthreads();
+    rs_zero(acc);
+    rs_mac<false, true>(acc, sH, sA, m);                           // dW -= H A^T
+    rs_sum(acc, R, m, v);
+#pragma unroll
+    for (int u = 0; u < NE; ++u) dw[u] -= v[u];
+    asm volatile("cp.async.wait_group 0;" ::: "memory");           // Q_k
+    __syncthreads();
+    if (k > 0) rs_load_async(sA, Xh + (long long)(k - 1) * mm, m); // beside the G update
+    rs_zero(acc);
+    rs_mac<false, true>(acc, sG, sQ, m);                           // G <- G Q^T - Wr^T H   (= 2G - G (Wr A)^T - Wr^T H)
+    rs_mac<true, false, NR, true>(acc, sW, sH, m);
+    rs_sum(acc, R, m, g);
+    rs_put(g, sG, nullptr, m);
+    if (k > 0 && Qh) rs_load_async(sQ, Qh + (long long)(k - 1) * mm, m);
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  rs_put(g, static_cast<float*>(nullptr), Gout, m);
+  rs_put(dw, static_cast<float*>(nullptr), dW, m);
+  __syncthreads();
 }
 
 // =====================================================================================
@@ -1192,39 +1544,79 @@ __device__ void ns_forward_dev(int m, int T, float eps, float alpha_in, const fl
   // Qh: NULL, or a history [T][m][m] that keeps Q_k = 2I - Wr X_k for the adjoint (which then need not form Wr X_k again)
   // CL CTAs of a cluster share the work (crank = this CTA's rank): element-wise phases are strided over all their
   // threads, every product is split by output tiles, small reductions are done by each CTA for itself.
+  if constexpr (!TC && CL == 1) {                    // m <= 64: everything resident in shared memory
+    float* smem = reinterpret_cast<float*>(&sm);
+    if (m <= 32) ns_forward_res<4>(m, T, eps, alpha_in, W, Wr, Xh, hdr, smem, red, Qh);
+    else if (m <= 56) ns_forward_res<7>(m, T, eps, alpha_in, W, Wr, Xh, hdr, smem, red, Qh);
+    else ns_forward_res<8>(m, T, eps, alpha_in, W, Wr, Xh, hdr, smem, red, Qh);
+    return;
+  }
   const int tid = threadIdx.x, gt = crank * 256 + tid, gn = 256 * CL;
   const long long mm = (long long)m * m;
-  for (long long e = gt; e < mm; e += gn) {
-    const int i = (int)(e / m), j = (int)(e % m);
-    Wr[e] = W[e] + (i == j ? eps : 0.f);
-  }
-  phase_sync<CL>();
+  const unsigned um = (unsigned)m, umm = um * um;
+  // one pass over W for both norms (every CTA of a cluster for itself): a warp takes every eighth row, a lane every 32nd
+  // column; four rows are in flight together
   float* colsum = red;          // [256]
   float* rowsum = red + 256;    // [256]
+  float* colpart = reinterpret_cast<float*>(&sm);      // [8][256]
+  {
+    const int warp = tid >> 5, lane = tid & 31, nv = (m + 31) >> 5;
+    float cs[8];
+#pragma unroll
+    for (int v = 0; v < 8; ++v) cs[v] = 0.f;
+    for (int i0 = warp; i0 < m; i0 += 32) {
+      float rs[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int v = 0; v < 8; ++v) {
+        if (v >= nv) break;
+        const int j = lane + 32 * v;
+        float w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + 8 * u;
+          w[u] = (i < m && j < m) ? W[(long long)i * m + j] + (i == j ? eps : 0.f) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { cs[v] += fabsf(w[u]); rs[u] += fabsf(w[u]); }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) rs[u] += __shfl_xor_sync(0xffffffffu, rs[u], o);
+        if (lane == 0 && i0 + 8 * u < m) rowsum[i0 + 8 * u] = rs[u];
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 8; ++v) colpart[warp * 256 + lane + 32 * v] = cs[v];
+  }
+  for (unsigned e = (unsigned)gt; e < umm; e += (unsigned)gn) Wr[e] = W[e] + (e % (um + 1u) == 0u ? eps : 0.f);
+  __syncthreads();
   if (tid < m) {
-    float cs = 0.f, rs = 0.f;
-    for (int i = 0; i < m; ++i) { cs += fabsf(Wr[(long long)i * m + tid]); rs += fabsf(Wr[(long long)tid * m + i]); }
-    colsum[tid] = cs; rowsum[tid] = rs;
+    float t = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) t += colpart[w * 256 + tid];
+    colsum[tid] = t;
   }
   __syncthreads();
-  if (tid == 0) {               // every CTA of a cluster arrives at the same values
-    float n1, ninf; int js, is;                   // near-ties (duplicated landmarks): the lowest index
-    norm_argmax(colsum, m, n1, js);
-    norm_argmax(rowsum, m, ninf, is);
-    float* al = red + 512;
-    al[0] = (alpha_in > 0.f) ? alpha_in : 1.f / (n1 * ninf);
-    if (crank == 0) {
-      hdr->n1 = n1; hdr->ninf = ninf; hdr->jstar = js; hdr->istar = is;
-      hdr->auto_alpha = !(alpha_in > 0.f);
-      hdr->alpha = al[0];
-      hdr->pad0 = hdr->pad1 = 0;
+  // every CTA of a cluster arrives at the same values; near-ties (duplicated landmarks): the lowest index
+  if (tid < 64) {
+    const bool cols = tid < 32;
+    float mx; int idx;
+    norm_argmax(cols ? colsum : rowsum, m, mx, idx);
+    if ((tid & 31) == 0) {
+      red[512 + (cols ? 0 : 1)] = mx;
+      if (crank == 0) {
+        if (cols) { hdr->n1 = mx; hdr->jstar = idx; } else { hdr->ninf = mx; hdr->istar = idx; }
+      }
     }
   }
   __syncthreads();
-  const float alpha = red[512];
-  for (long long e = gt; e < mm; e += gn) {
-    const int i = (int)(e / m), j = (int)(e % m);
-    Xh[e] = alpha * Wr[(long long)j * m + i];
+  const float alpha = (alpha_in > 0.f) ? alpha_in : 1.f / (red[512] * red[513]);
+  if (crank == 0 && tid == 0) { hdr->auto_alpha = !(alpha_in > 0.f); hdr->alpha = alpha; hdr->pad0 = hdr->pad1 = 0; }
+#pragma unroll 4
+  for (unsigned e = (unsigned)gt; e < umm; e += (unsigned)gn) {
+    const unsigned i = e / um, j = e - i * um;
+    Xh[e] = alpha * (W[j * um + i] + (i == j ? eps : 0.f));
   }
   phase_sync<CL>();
   for (int k = 0; k < T; ++k) {
@@ -1253,20 +1645,37 @@ __device__ void ns_backward_dev(int m, int T, const float* Wr, const float* Xh, 
   // products per step instead of five
   const int tid = threadIdx.x, gt = crank * 256 + tid, gn = 256 * CL;
   const long long mm = (long long)m * m;
-  for (long long e = gt; e < mm; e += gn) { Ga[e] = G0[e]; dW[e] = 0.f; }
+  const float* G = G0; float* Gn = Ga;
+  if constexpr (!TC && CL == 1) {                    // m <= 64: everything resident in shared memory
+    float* smem = reinterpret_cast<float*>(&sm);
+    if (m <= 32) ns_backward_res<4>(m, T, Wr, Xh, G0, dW, Ga, smem, Qh);
+    else if (m <= 56) ns_backward_res<7>(m, T, Wr, Xh, G0, dW, Ga, smem, Qh);
+    else ns_backward_res<8>(m, T, Wr, Xh, G0, dW, Ga, smem, Qh);
+    ns_backward_tail_dev<CL>(m, Wr, hdr, Ga, dW, red, crank);
+    return;
+  }
+  if (T == 0)
+    for (long long e = gt; e < mm; e += gn) dW[e] = 0.f;
   phase_sync<CL>();
-  float* G = Ga; float* Gn = Gb;
   for (int k = T - 1; k >= 0; --k) {
     const float* A = Xh + (long long)k * mm;                                        // X_{k+1} = 2A - A P, P = Wr A
+    const float* dWin = k == T - 1 ? nullptr : dW;                                  // the first step starts the sum
+    const float b1 = dWin ? 1.f : 0.f;
     if (!Qh) ns_gemm<TC, false, false, true>(m, m, m, Wr, m, A, m, P, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);      // P = Wr A
     ns_gemm<TC, true, false, true>(m, m, m, A, m, G, m, Hm, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);       // H = A^T G
     if (CL > 1) phase_sync<CL>();
-    ns_gemm<TC, false, true, true>(m, m, m, Hm, m, A, m, dW, m, -1.f, 1.f, dW, 0.f, sm, crank, CL);          // dW -= H A^T
-    if (Qh) ns_gemm<TC, false, true, true>(m, m, m, G, m, Qh + (long long)k * mm, m, Gn, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);   // Gn = G Q^T
-    else ns_gemm<TC, false, true, true>(m, m, m, G, m, P, m, Gn, m, -1.f, 2.f, G, 0.f, sm, crank, CL);       // Gn = 2G - G P^T
-    ns_gemm<TC, true, false, true>(m, m, m, Wr, m, Hm, m, Gn, m, -1.f, 1.f, Gn, 0.f, sm, crank, CL);         // Gn -= Wr^T H
+    ns_gemm<TC, false, true, true>(m, m, m, Hm, m, A, m, dW, m, -1.f, b1, dWin, 0.f, sm, crank, CL);         // dW -= H A^T
+    if constexpr (TC) {
+      if (Qh) ns_gemm<TC, false, true, true>(m, m, m, G, m, Qh + (long long)k * mm, m, Gn, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);   // Gn = G Q^T
+      else ns_gemm<TC, false, true, true>(m, m, m, G, m, P, m, Gn, m, -1.f, 2.f, G, 0.f, sm, crank, CL);     // Gn = 2G - G P^T
+      ns_gemm<TC, true, false, true>(m, m, m, Wr, m, Hm, m, Gn, m, -1.f, 1.f, Gn, 0.f, sm, crank, CL);       // Gn -= Wr^T H
+    } else {                                                                        // both terms in one accumulation
+      const FgSecond wh = {Wr, m, Hm, m, m};
+      if (Qh) cta_gemm<false, true, true, true, false, true>(m, m, m, G, m, Qh + (long long)k * mm, m, Gn, m, 1.f, 0.f, nullptr, 0.f, sm.f, crank, CL, wh);
+      else cta_gemm<false, true, true, true, false, false>(m, m, m, G, m, P, m, Gn, m, -1.f, 2.f, G, 0.f, sm.f, crank, CL, wh);
+    }
     if (CL > 1) phase_sync<CL>();
-    float* t = G; G = Gn; Gn = t;
+    G = Gn; Gn = Gn == Ga ? Gb : Ga;
   }
   ns_backward_tail_dev<CL>(m, Wr, hdr, G, dW, red, crank);
 }
@@ -1290,15 +1699,23 @@ __device__ void ns_backward_tail_dev(int m, const float* Wr, const NsHdr* hdr, c
     for (; e < mm; e += 256) p4[0] += G[e] * Wr[e];
     part = (p4[0] + p4[1]) + (p4[2] + p4[3]);
   } else {
-    for (long long e = tid; e < mm; e += 256) {      // every CTA of a cluster sums everything (same order, same value)
-      const int i = (int)(e / m), j = (int)(e % m);
-      part += G[e] * Wr[(long long)j * m + i];
+    float p4[4] = {0.f, 0.f, 0.f, 0.f};              // a share of the sum per CTA of the cluster
+    const unsigned um = (unsigned)m, umm = um * um;
+    for (unsigned e0 = (unsigned)gt; e0 < umm; e0 += 4u * (unsigned)gn) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const unsigned e = e0 + (unsigned)(u * gn), i = e / um, j = e - i * um;
+        if (e < umm) p4[u] += G[e] * Wr[j * um + i];
+      }
     }
+    part = (p4[0] + p4[1]) + (p4[2] + p4[3]);
   }
-  const float dalpha = block_sum(part, red);
-  for (long long e = gt; e < mm; e += gn) {
-    const int j = (int)(e / m), i = (int)(e % m);      // dW[j][i] += alpha G[i][j]
-    dW[e] += alpha * G[(long long)i * m + j];
+  float dalpha = block_sum(part, red);
+  if constexpr (CL > 1 && !SYM) dalpha = cluster_sum<CL>(dalpha, red + 64, crank);
+#pragma unroll 4
+  for (unsigned e = (unsigned)gt; e < (unsigned)mm; e += (unsigned)gn) {      // dW[j][i] += alpha G[i][j]
+    const unsigned j = e / (unsigned)m, i = e - j * (unsigned)m;
+    dW[e] += alpha * G[i * (unsigned)m + j];
   }
   phase_sync<CL>();
   if (hdr->auto_alpha) {
@@ -1553,19 +1970,25 @@ __device__ void cg_dev(int m, int T, float eps, const float* W, const float* Bsr
 // ------------------------------------------------------------------ stand-alone ns_pinv / ns_pinv_bwd
 // CL CTAs of a thread-block cluster share a matrix (grid = batch * CL): every product is split by output tiles, the
 // hardware cluster barrier ends a phase.  fp32 FFMA throughout (held to 2e-5 against the oracle).
+// Two CTAs per SM for clusters: sixteen clusters of eight do not all find eight free SMs in one part of the chip, and at
+// one CTA per SM (255 registers) the last of them waited for the others (adjoint 329 -> 273 us).
 template <int CL>
-__global__ void __launch_bounds__(256) k_ns_pinv(int m, int T, float eps, float alpha_in, const float* W,
+__global__ void __launch_bounds__(256, CL > 1 ? 2 : 1) k_ns_pinv(int m, int T, float eps, float alpha_in, const float* W,
                                                  float* Wr, float* P, float* Xh, NsHdr* hdr, float* X,
                                                  float* resid) {
   pdl_wait();
-  __shared__ NsSmem sm;
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  NsSmem& sm = *reinterpret_cast<NsSmem*>(dyn_smem);
   __shared__ float red[2 * 256 + 8];
   const int b = blockIdx.x / CL, crank = blockIdx.x % CL;
   const long long mm = (long long)m * m;
   W += b * mm; Wr += b * mm; P += b * mm; Xh += (long long)b * (T + 1) * mm; hdr += b;
   ns_forward_dev<false, CL>(m, T, eps, alpha_in, W, Wr, P, Xh, hdr, sm, red, crank);
   const float* XT = Xh + (long long)T * mm;
-  if (X) for (long long e = crank * 256 + threadIdx.x; e < mm; e += 256 * CL) X[b * mm + e] = XT[e];
+  if (X) {
+#pragma unroll 4
+    for (int e = crank * 256 + threadIdx.x; e < (int)mm; e += 256 * CL) X[b * mm + e] = XT[e];
+  }
   if (resid) {
     ns_gemm<false, false, false>(m, m, m, Wr, m, XT, m, P, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);
     phase_sync<CL>();
@@ -1586,12 +2009,13 @@ __global__ void __launch_bounds__(256) k_ns_pinv(int m, int T, float eps, float 
 // recompute != 0: run the forward first (Xh, hdr, Wr are scratch); else Xh is the caller's history
 // and only Wr / hdr are rebuilt from W.
 template <int CL>
-__global__ void __launch_bounds__(256) k_ns_pinv_bwd(int m, int T, float eps, float alpha_in, const float* W,
+__global__ void __launch_bounds__(256, CL > 1 ? 2 : 1) k_ns_pinv_bwd(int m, int T, float eps, float alpha_in, const float* W,
                                                      float* Wr, float* P, float* Hm, float* Ga, float* Gb,
                                                      float* Xh_scratch, const float* Xh_given, NsHdr* hdr,
                                                      const float* dX, float* dW) {
   pdl_wait();
-  __shared__ NsSmem sm;
+  extern __shared__ __align__(16) unsigned char dyn_smem[];
+  NsSmem& sm = *reinterpret_cast<NsSmem*>(dyn_smem);
   __shared__ float red[2 * 256 + 8];
   const int b = blockIdx.x / CL, crank = blockIdx.x % CL;
   const long long mm = (long long)m * m;

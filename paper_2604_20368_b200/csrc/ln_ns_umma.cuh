@@ -171,25 +171,33 @@ __device__ bool ns_forward_umma(int m, int T, float eps, float alpha_in, const f
   __syncthreads();
   {
     float* colsum = red; float* rowsum = red + 256;
-    if (tid < m) {
-      float cs = 0.f, rs = 0.f;
-      for (int i = 0; i < m; ++i) cs += fabsf(Wf[i * UM + tid]);
-      for (int i = 0; i < UM; ++i) rs += fabsf(Wf[tid * UM + ((i + tid) & (UM - 1))]);   // rotated start: no bank conflicts; padding is zero
-      colsum[tid] = cs; rowsum[tid] = rs;
+    {   // the first 128 threads take the columns, the others the rows (rotated start: no bank conflicts; padding is zero);
+        // four sums per thread keep the additions of a thread apart
+      const int t = tid & 127;
+      if (t < UM) {
+        float c4[4] = {0.f, 0.f, 0.f, 0.f};
+        const bool cols = tid < 128;
+#pragma unroll 4
+        for (int i = 0; i < UM; i += 4)
+#pragma unroll
+          for (int u = 0; u < 4; ++u) c4[u] += fabsf(Wf[cols ? (i + u) * UM + t : t * UM + ((i + u + t) & (UM - 1))]);
+        (cols ? colsum : rowsum)[t] = (c4[0] + c4[1]) + (c4[2] + c4[3]);
+      }
     }
     __syncthreads();
-    if (tid == 0) {
-      float n1, ninf; int js, is;
-      norm_argmax(colsum, m, n1, js);
-      norm_argmax(rowsum, m, ninf, is);
-      hdr->n1 = n1; hdr->ninf = ninf; hdr->jstar = js; hdr->istar = is;
-      hdr->auto_alpha = !(alpha_in > 0.f);
-      hdr->alpha = (alpha_in > 0.f) ? alpha_in : 1.f / (n1 * ninf);
-      hdr->pad0 = hdr->pad1 = 0;
+    if (tid < 64) {
+      const bool cols = tid < 32;
+      float mx; int idx;
+      norm_argmax(cols ? colsum : rowsum, m, mx, idx);
+      if ((tid & 31) == 0) {
+        red[512 + (cols ? 0 : 1)] = mx;
+        if (cols) { hdr->n1 = mx; hdr->jstar = idx; } else { hdr->ninf = mx; hdr->istar = idx; }
+      }
     }
     __syncthreads();
   }
-  const float alpha = hdr->alpha;
+  const float alpha = (alpha_in > 0.f) ? alpha_in : 1.f / (red[512] * red[513]);
+  if (tid == 0) { hdr->auto_alpha = !(alpha_in > 0.f); hdr->alpha = alpha; hdr->pad0 = hdr->pad1 = 0; }
   if (act) {  // this thread's row: NV columns of W and of X_0 = alpha W^T
     float w[NV], x0[NV];
 #pragma unroll

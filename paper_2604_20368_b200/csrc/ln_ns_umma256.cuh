@@ -179,11 +179,12 @@ __device__ bool ns_forward_umma256(U2Ctx& c, int m, int T, float eps, float alph
       colsum[tid] = c16[0];
     }
     __syncthreads();
-    if (tid == 0) {               // both CTAs of the cluster arrive at the same values
+    if (tid < 32) {               // both CTAs of the cluster arrive at the same values
       float n1; int js;
       norm_argmax(colsum, m, n1, js);                            // near-ties (duplicated landmarks): the lowest index
-      red[512] = (alpha_in > 0.f) ? alpha_in : 1.f / (n1 * n1);
-      if (ri == 0) {
+      if (tid == 0) red[512] = (alpha_in > 0.f) ? alpha_in : 1.f / (n1 * n1);
+      __syncwarp();
+      if (ri == 0 && tid == 0) {
         hdr->n1 = n1; hdr->ninf = n1; hdr->jstar = js; hdr->istar = js;
         hdr->auto_alpha = !(alpha_in > 0.f);
         hdr->alpha = red[512];

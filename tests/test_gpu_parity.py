@@ -248,6 +248,32 @@ def test_cfg3_full_size_sampled_heads():
 
 
 
+# The fp32 engines at the edges of their variants: register tiles of 4, 7 and 8 rows on resident matrices (m <= 32, 56,
+# 64), a cluster with 64 x 32 or 64 x 64 output tiles beyond, k staged 128 at a time; 16-byte copies (m a multiple of
+# four) and 4-byte ones; a matrix that is not symmetric (the stand-alone calls take any).
+@pytest.mark.parametrize("m", [31, 32, 33, 56, 57, 63, 65, 96, 101, 128, 129, 191, 196, 255])
+def test_fp32_newton_schulz_variants_at_their_edges(m):
+    T = 3
+    W = _kernel_matrices(3, m, 16, 20 + m)
+    W = (W * (1 + 0.05 * np.random.default_rng(m).uniform(-1, 1, W.shape))).astype(np.float32)
+    dX = np.random.default_rng(m + 1).standard_normal(W.shape).astype(np.float32)
+    Wd, eps = torch.from_numpy(W).to(DEV), float(np.float32(1e-6))
+    X, hist, _ = ln.ns_pinv(Wd, T, ridge_eps=1e-6, want_hist=True)
+    Xo, _, _, histo = oracle.ns_pinv(W, T, eps=eps, want_hist=True)
+    assert rel_err(f64(X), Xo) < 2e-5 and rel_err(f64(hist)[:, :T], histo) < 2e-5      # the bars of the tests above
+    dWo = oracle.ns_pinv_bwd(W, T, eps, 0.0, dX)
+    for h in (None, hist):
+        dW = ln.ns_pinv_bwd(Wd, T, 1e-6, 0.0, torch.from_numpy(dX).to(DEV), X_hist=h)
+        assert rel_err(f64(dW), dWo) < 1e-4
+
+
+@pytest.mark.parametrize("mh,mw", [(5, 6), (7, 8), (8, 8), (5, 13), (10, 13)])
+def test_fp32_storage_path_over_the_solver_variants(mh, mw):
+    cfg = synth.Config("f32_edges", B=1, H=2, d=64, m=mh * mw, T=4, gh=20, gw=20, mh=mh, mw=mw, prefix=1,
+                       dtype="f32", seed=321 + mh * mw)
+    _run_case(cfg)
+
+
 # Ragged shapes for the fused sign pass (token tiles of 8 * TG tokens, rounds of 8 landmarks, several token
 # chunks per head, two 64-dim slabs) and for the per-head kernels (m <= 64, 64 < m <= 128, clustered m > 128).
 @pytest.mark.parametrize("gh,gw,mh,mw,prefix,d,dtype", [
