@@ -84,19 +84,30 @@ __global__ void __launch_bounds__(256, 3) k_nn_umma(const float* __restrict__ E,
   __syncthreads();
   umma::fence_after_sync();
   const uint32_t tacc = tmem_base;
-  // E block: thread = (token r of the tile, 32 landmarks of the block)
-  const int zr = tid >> 1, zc = (tid & 1) * 32, zi = i0 + zr;
-  const bool in = zi < n;
-  const float mi = (mu && in) ? mu[(long long)bh * n + zi] : 0.f;
+  // E block: a warp takes pieces of 8 rows x 32 landmarks, lane = (row % 8, eight landmarks): its loads touch eight lines of
+  // 128 contiguous bytes, and the eight lanes of a shared-memory phase write the eight rows of one core matrix.  (With a
+  // row half per thread every lane of a load touched a line of its own: O / dV at 128 heads x 4096 tokens x 256 landmarks,
+  // 128 dims 240 / 224 -> 219 / 205 us.)
+  const int lane = tid & 31, zr = 8 * (warp >> 1) + (lane & 7), zc = 32 * (warp & 1) + 8 * (lane >> 3);
+  float mi[4];
+  bool in[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int zi = i0 + zr + 32 * u;
+    in[u] = zi < n;
+    mi[u] = (mu && in[u]) ? mu[(long long)bh * n + zi] : 0.f;
+  }
+  const float* const Erow = E + (long long)(i0 + zr) * lde + zc;
   const uint32_t idesc = umma::instr_desc(D, false, true);
   uint32_t ph_mma = 0, ph_y = 0;
   bool ok = true;
-  float4 v[8];                                   // this thread's piece of an E block, fetched one block ahead
+  float4 v[8];                                   // this thread's pieces of an E block, fetched one block ahead
   auto fetch = [&](int kb) {
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const int l = kb * GU_KB + zc + 4 * q;
-      v[q] = (in && l < m) ? *reinterpret_cast<const float4*>(E + (long long)zi * lde + l) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const int l = kb * GU_KB + zc + 4 * (q & 1);
+      v[q] = (in[q >> 1] && l < m) ? *reinterpret_cast<const float4*>(Erow + (long long)(32 * (q >> 1)) * lde + kb * GU_KB + 4 * (q & 1))
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
   fetch(0);
@@ -106,16 +117,16 @@ __global__ void __launch_bounds__(256, 3) k_nn_umma(const float* __restrict__ E,
       umma::bulk_load(sY, Yimg + (long long)kb * (2 * GU_KB * D), 2 * GU_KB * D * 2, &mbar_y);
     }
 #pragma unroll
-    for (int q = 0; q < 8; q += 2) {
-      float4 a = v[q], b = v[q + 1];
-      const int l = kb * GU_KB + zc + 4 * q;
-      a.x = (in && l < m) ? a.x - mi : 0.f;     a.y = (in && l + 1 < m) ? a.y - mi : 0.f;
-      a.z = (in && l + 2 < m) ? a.z - mi : 0.f; a.w = (in && l + 3 < m) ? a.w - mi : 0.f;
-      b.x = (in && l + 4 < m) ? b.x - mi : 0.f; b.y = (in && l + 5 < m) ? b.y - mi : 0.f;
-      b.z = (in && l + 6 < m) ? b.z - mi : 0.f; b.w = (in && l + 7 < m) ? b.w - mi : 0.f;
+    for (int u = 0; u < 4; ++u) {
+      float4 a = v[2 * u], b = v[2 * u + 1];
+      const int l = kb * GU_KB + zc;
+      a.x = (in[u] && l < m) ? a.x - mi[u] : 0.f;     a.y = (in[u] && l + 1 < m) ? a.y - mi[u] : 0.f;
+      a.z = (in[u] && l + 2 < m) ? a.z - mi[u] : 0.f; a.w = (in[u] && l + 3 < m) ? a.w - mi[u] : 0.f;
+      b.x = (in[u] && l + 4 < m) ? b.x - mi[u] : 0.f; b.y = (in[u] && l + 5 < m) ? b.y - mi[u] : 0.f;
+      b.z = (in[u] && l + 6 < m) ? b.z - mi[u] : 0.f; b.w = (in[u] && l + 7 < m) ? b.w - mi[u] : 0.f;
       uint2 h0, l0, h1, l1;
       split4(a, h0, l0); split4(b, h1, l1);
-      const int off = umma::img(zr, zc + 4 * q, GU_KB);
+      const int off = umma::img(zr + 32 * u, zc, GU_KB);
       *reinterpret_cast<uint4*>(sZ + off) = make_uint4(h0.x, h0.y, h1.x, h1.y);
       *reinterpret_cast<uint4*>(sZ + 128 * GU_KB + off) = make_uint4(l0.x, l0.y, l1.x, l1.y);
     }

@@ -160,8 +160,12 @@ __global__ void __launch_bounds__(256, 2) k_sign3(const bf16* __restrict__ tok, 
     const bf16* Yh = Yimg + (long long)bh * nkb * (2 * GU_KB * D);
     if (umma::leader(tid)) { umma::mbar_expect_tx(&mbar_y, YB); umma::bulk_load(sY, Yh, YB, &mbar_y); }
     const bf16* Uh = U + (long long)bh * n * D;
-    for (int p = tid; p < 128 * (D / 8); p += nthr) {
-      const int r = p / (D / 8), c8 = (p % (D / 8)) * 8;
+    // a warp copies pieces of 8 rows x 32 dims, lane = (row % 8, eight dims): whole 32-byte sectors from global memory, and
+    // the eight lanes of a shared-memory phase write the eight rows of one core matrix (no bank conflicts; with the lanes
+    // along a row every phase hit one bank group eight times: DeiT-shaped pass 98.6 -> 96.7 us)
+#pragma unroll 4
+    for (int p = warp; p < 16 * (D / 32); p += nwarps) {
+      const int r = 8 * (p / (D / 32)) + (lane & 7), c8 = 32 * (p % (D / 32)) + 8 * (lane >> 3);
       uint4 v = make_uint4(0u, 0u, 0u, 0u);
       if (i0 + r < n && r < TT8) v = *reinterpret_cast<const uint4*>(Uh + (long long)(i0 + r) * D + c8);
       *reinterpret_cast<uint4*>(sU + umma::img(r, c8, D)) = v;
