@@ -801,8 +801,8 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
   }
   if (sign3) {
     const long long cnt = (long long)BH * m * D;
-    LN_LAUNCH("k_fold_landmarks", st, enqueue(k_fold_landmarks, cdiv(cnt, 256), 256, 0, st, LfC, w.SB, D, cnt));
-    if (two) LN_LAUNCH("k_fold_landmarks", st, enqueue(k_fold_landmarks, cdiv(cnt, 256), 256, 0, st, LfR, w.SBq, D, cnt));
+    LN_LAUNCH("k_fold_landmarks", st, enqueue(k_fold_landmarks, cdiv(cnt / 4, 256), 256, 0, st, LfC, w.SB, D == 128 ? 5 : 4, cnt / 4));
+    if (two) LN_LAUNCH("k_fold_landmarks", st, enqueue(k_fold_landmarks, cdiv(cnt / 4, 256), 256, 0, st, LfR, w.SBq, D == 128 ? 5 : 4, cnt / 4));
     if (qrows_f) launch_sign3("sign3_dQ_dLC", Q, dO, x.Yimg, x.C, qrows_f, w.dLCpart, w.SB, kap);
     else launch_sign3("sign3_dQ_dLC", Q, dO, x.Yimg, x.C, dQ, w.dLCpart, w.SB, kap);
   } else {

@@ -371,6 +371,18 @@ template <typename T> __global__ void k_to_f32(const T* __restrict__ x, float* _
 // =====================================================================================
 // filt: NULL = average pooling; else the depth-wise-convolution selection of Sec. 4.2, one filter per head and channel,
 // [H][taps][d] with taps = (gh/mh) * (gw/mw) (the grid divides: the host checks), tap (u, v) of a region at u (gw/mw) + v
+// four consecutive elements as they lie in memory, and as fp32
+template <typename T> struct Raw4;
+template <> struct Raw4<float> {
+  typedef float4 type;
+  __device__ static __forceinline__ float4 f(const float4& v) { return v; }
+};
+template <> struct Raw4<bf16> {
+  typedef uint2 type;
+  __device__ static __forceinline__ float4 f(const uint2& r) {
+    return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16), __uint_as_float(r.y & 0xffff0000u));
+  }
+};
 struct PoolGeom { int n, d, m, prefix, gh, gw, mh, mw; const float* filt; int H; };
 // 32-bit on purpose (64-bit division costs two orders of magnitude more on the device); the host
 // checks that gh * mh and gw * mw stay below 2^31.
@@ -393,14 +405,35 @@ __global__ void __launch_bounds__(256) k_pool(const T* __restrict__ K, float* __
   // depend on the order of a single-precision summation.
   double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
   const float* wf = g.filt ? g.filt + (long long)(bh % g.H) * ((r1 - r0) * (c1 - c0)) * g.d + c : nullptr;
-  for (int r = r0; r < r1; ++r)
-    for (int q = c0; q < c1; ++q) {
-      const float4 v = ld4(Kh + (long long)(g.prefix + r * g.gw + q) * g.d + c);
-      if (wf) {                        // products of an fp32 weight and a token value are exact in double
-        const float4 w = ld4(wf + (long long)((r - r0) * (c1 - c0) + (q - c0)) * g.d);
-        s0 += (double)w.x * (double)v.x; s1 += (double)w.y * (double)v.y; s2 += (double)w.z * (double)v.z; s3 += (double)w.w * (double)v.w;
-      } else { s0 += (double)v.x; s1 += (double)v.y; s2 += (double)v.z; s3 += (double)v.w; }
+  auto add = [&](const float4& f, int t) {
+    if (wf) {                          // products of an fp32 weight and a token value are exact in double
+      const float4 w = ld4(wf + (long long)t * g.d);
+      s0 += (double)w.x * (double)f.x; s1 += (double)w.y * (double)f.y; s2 += (double)w.z * (double)f.z; s3 += (double)w.w * (double)f.w;
+    } else { s0 += (double)f.x; s1 += (double)f.y; s2 += (double)f.z; s3 += (double)f.w; }
+  };
+  const int ntok = (r1 - r0) * (c1 - c0);
+  const T* row = Kh + (long long)(g.prefix + r0 * g.gw) * g.d + c;
+  if (ntok <= 8) {
+    for (int t = 0, r = r0; r < r1; ++r, row += (long long)g.gw * g.d)
+      for (int q = c0; q < c1; ++q, ++t) add(ld4(row + (long long)q * g.d), t);
+  } else {
+    // Eight tokens of the bin in flight, added in their order: with 7 x 7-token bins at 32 heads x 3136 tokens 23.7 ->
+    // 17.3 us, with 4 x 4 in fp32 at 32 heads x 784 13.8 -> 9.2 us.  Up to eight tokens the loads are too few for the
+    // bookkeeping to pay (2 x 2 bins at 384 heads x 197: 14.1 against 16.6 us).
+    for (int t0 = 0, q = c0; t0 < ntok; t0 += 8) {
+      typename Raw4<T>::type v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (t0 + u < ntok) v[u] = *reinterpret_cast<const typename Raw4<T>::type*>(row + (long long)q * g.d);
+        if (++q == c1) { q = c0; row += (long long)g.gw * g.d; }
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (t0 + u >= ntok) break;
+        add(Raw4<T>::f(v[u]), t0 + u);
+      }
     }
+  }
   const double cnt = wf ? 1.0 : (double)((r1 - r0) * (c1 - c0));
   st4(L + ((long long)bh * g.m + l) * g.d + c,
       make_float4((float)(s0 / cnt), (float)(s1 / cnt), (float)(s2 / cnt), (float)(s3 / cnt)));

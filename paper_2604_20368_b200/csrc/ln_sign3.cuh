@@ -46,15 +46,19 @@ static_assert((size_t)(128 * 128 + 2 * GU_KB * 128) * sizeof(bf16) <= sizeof(flo
               "the operand images of the MMA phase fit in the column-partial buffers they alias");
 
 // Scale and offset of every landmark value (see fold_pair): SB[bh][j][0][c] = s, SB[bh][j][1][c] = b.
-__global__ void __launch_bounds__(256) k_fold_landmarks(const float* __restrict__ Lm, float* __restrict__ SB, int D, long long count) {
+// Four dims per thread, D a power of two (64 or 128): log2q = log2(D / 4).  Bound by memory; with one element and a 64-bit
+// division per thread 20.0 us where it takes 11.7 (128 heads x 256 landmarks, 128 dims).
+__global__ void __launch_bounds__(256) k_fold_landmarks(const float* __restrict__ Lm, float* __restrict__ SB, int log2q, long long quads) {
   pdl_wait();
-  const long long e = (long long)blockIdx.x * 256 + threadIdx.x;     // index into Lm [BH * m][D]
-  if (e >= count) return;
-  const long long row = e / D; const int c = (int)(e % D);
-  float s, b;
-  fold_pair(Lm[e], s, b);
-  SB[(row * 2) * D + c] = s;
-  SB[(row * 2 + 1) * D + c] = b;
+  const long long e = (long long)blockIdx.x * 256 + threadIdx.x;     // quad of Lm [BH * m][D]
+  if (e >= quads) return;
+  const long long row = e >> log2q;
+  const int c = (int)(e & ((1 << log2q) - 1)) * 4, D = 4 << log2q;
+  const float4 y = ld4(Lm + 4 * e);
+  float4 s, b;
+  fold_pair(y.x, s.x, b.x); fold_pair(y.y, s.y, b.y); fold_pair(y.z, s.z, b.z); fold_pair(y.w, s.w, b.w);
+  st4(SB + row * 2 * D + c, s);
+  st4(SB + (row * 2 + 1) * D + c, b);
 }
 
 __device__ __forceinline__ void s3_cp_async16(void* dst_smem, const void* src, bool valid) {

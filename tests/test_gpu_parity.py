@@ -93,6 +93,25 @@ def test_l1_kernel_bwd(batch, na, nb, d, dtype, recompute):
     assert rel_err(f64(dB), dBo) < tol
 
 
+@pytest.mark.parametrize("gh,gw,mh,mw,prefix", [(8, 8, 4, 4, 0), (9, 8, 3, 4, 1), (12, 9, 4, 3, 1), (16, 16, 4, 4, 0),
+                                                (29, 21, 4, 3, 1), (7, 63, 1, 1, 0)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_landmarks_pool_bin_sizes(gh, gw, mh, mw, prefix, dtype):
+    """Bins of 4, 6 to 9, 9, 16, 56 to 64 (overlapping) and 441 tokens: below, at and above the eight tokens from which
+    the loads are batched, and the kernel for large bins.  A landmark is the fp32 value nearest to the exact mean."""
+    n, d = prefix + gh * gw, 64
+    K = _rand((2, 3, n, d), 31, dtype)
+    p = ln.problem_from_config(synth.Config("bins", B=2, H=3, d=d, m=mh * mw, T=1, gh=gh, gw=gw, mh=mh, mw=mw, prefix=prefix,
+                                            dtype="f32" if dtype == torch.float32 else "bf16", seed=1), whiten=None)
+    L = ln.landmarks_pool(p, K.to(DEV))
+    G = f64(K)[:, :, prefix:].reshape(2, 3, gh, gw, d)
+    lo, hi = lambda a, g, m: a * g // m, lambda a, g, m: -(-(a + 1) * g // m)
+    ref = np.stack([G[:, :, lo(a, gh, mh):hi(a, gh, mh), lo(b, gw, mw):hi(b, gw, mw)].mean(axis=(2, 3))
+                    for a in range(mh) for b in range(mw)], axis=2)
+    # one rounding to fp32 (2^-24 relative), and numpy's own mean in double
+    assert np.abs(f64(L).reshape(ref.shape) - ref).max() <= 2.0 ** -23 * np.abs(ref).max()
+
+
 # ------------------------------------------------------------------------------------------ ns_pinv
 def _kernel_matrices(batch, m, d, seed):
     pts = np.random.default_rng(seed).standard_normal((batch, m, d))
