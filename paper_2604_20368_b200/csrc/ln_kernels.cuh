@@ -1587,48 +1587,64 @@ __device__ void ns_forward_dev(int m, int T, float eps, float alpha_in, const fl
   const int tid = threadIdx.x, gt = crank * 256 + tid, gn = 256 * CL;
   const long long mm = (long long)m * m;
   const unsigned um = (unsigned)m, umm = um * um;
-  // one pass over W for both norms (every CTA of a cluster for itself): a warp takes every eighth row, a lane every 32nd
-  // column; four rows are in flight together
+  // both norms, every CTA of a cluster for itself
   float* colsum = red;          // [256]
   float* rowsum = red + 256;    // [256]
-  float* colpart = reinterpret_cast<float*>(&sm);      // [8][256]
-  {
-    const int warp = tid >> 5, lane = tid & 31, nv = (m + 31) >> 5;
-    float cs[8];
-#pragma unroll
-    for (int v = 0; v < 8; ++v) cs[v] = 0.f;
-    for (int i0 = warp; i0 < m; i0 += 32) {
-      float rs[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int v = 0; v < 8; ++v) {
-        if (v >= nv) break;
-        const int j = lane + 32 * v;
-        float w[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int i = i0 + 8 * u;
-          w[u] = (i < m && j < m) ? W[(long long)i * m + j] + (i == j ? eps : 0.f) : 0.f;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { cs[v] += fabsf(w[u]); rs[u] += fabsf(w[u]); }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) rs[u] += __shfl_xor_sync(0xffffffffu, rs[u], o);
-        if (lane == 0 && i0 + 8 * u < m) rowsum[i0 + 8 * u] = rs[u];
+  for (unsigned e = (unsigned)gt; e < umm; e += (unsigned)gn) Wr[e] = W[e] + (e % (um + 1u) == 0u ? eps : 0.f);
+  if constexpr (TC) {
+    // One chain of additions per sum, in index order: the scale of X_0, and with it the bits of every bf16 output, hangs
+    // on it.  Up to 128 columns half of the threads take the rows beside the other half's columns.
+    const int mp = m <= 128 ? 128 : 256;
+    for (int s = tid; s < 2 * mp; s += 256) {
+      const bool cols = s < mp;
+      const int t = cols ? s : s - mp;
+      float sum = 0.f;
+      if (t < m) {
+#pragma unroll 8
+        for (int i = 0; i < m; ++i) sum += fabsf(W[cols ? i * m + t : t * m + i] + (i == t ? eps : 0.f));
+        (cols ? colsum : rowsum)[t] = sum;
       }
     }
+  } else {
+    // one pass over W: a warp takes every eighth row, a lane every 32nd column; four rows are in flight together
+    float* colpart = reinterpret_cast<float*>(&sm);      // [8][256]
+    {
+      const int warp = tid >> 5, lane = tid & 31, nv = (m + 31) >> 5;
+      float cs[8];
 #pragma unroll
-    for (int v = 0; v < 8; ++v) colpart[warp * 256 + lane + 32 * v] = cs[v];
-  }
-  for (unsigned e = (unsigned)gt; e < umm; e += (unsigned)gn) Wr[e] = W[e] + (e % (um + 1u) == 0u ? eps : 0.f);
-  __syncthreads();
-  if (tid < m) {
-    float t = 0.f;
+      for (int v = 0; v < 8; ++v) cs[v] = 0.f;
+      for (int i0 = warp; i0 < m; i0 += 32) {
+        float rs[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int w = 0; w < 8; ++w) t += colpart[w * 256 + tid];
-    colsum[tid] = t;
+        for (int v = 0; v < 8; ++v) {
+          if (v >= nv) break;
+          const int j = lane + 32 * v;
+          float w[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int i = i0 + 8 * u;
+            w[u] = (i < m && j < m) ? W[(long long)i * m + j] + (i == j ? eps : 0.f) : 0.f;
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) { cs[v] += fabsf(w[u]); rs[u] += fabsf(w[u]); }
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) rs[u] += __shfl_xor_sync(0xffffffffu, rs[u], o);
+          if (lane == 0 && i0 + 8 * u < m) rowsum[i0 + 8 * u] = rs[u];
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < 8; ++v) colpart[warp * 256 + lane + 32 * v] = cs[v];
+    }
+    __syncthreads();
+    if (tid < m) {
+      float t = 0.f;
+#pragma unroll
+      for (int w = 0; w < 8; ++w) t += colpart[w * 256 + tid];
+      colsum[tid] = t;
+    }
   }
   __syncthreads();
   // every CTA of a cluster arrives at the same values; near-ties (duplicated landmarks): the lowest index
@@ -1663,7 +1679,7 @@ __device__ void ns_forward_dev(int m, int T, float eps, float alpha_in, const fl
   }
 }
 
-template <int CL, bool SYM = false>
+template <bool TC, int CL>
 __device__ void ns_backward_tail_dev(int m, const float* Wr, const NsHdr* hdr, const float* G, float* dW, float* red, int crank);
 
 // =====================================================================================
@@ -1684,7 +1700,7 @@ __device__ void ns_backward_dev(int m, int T, const float* Wr, const float* Xh, 
     if (m <= 32) ns_backward_res<4>(m, T, Wr, Xh, G0, dW, Ga, smem, Qh);
     else if (m <= 56) ns_backward_res<7>(m, T, Wr, Xh, G0, dW, Ga, smem, Qh);
     else ns_backward_res<8>(m, T, Wr, Xh, G0, dW, Ga, smem, Qh);
-    ns_backward_tail_dev<CL>(m, Wr, hdr, Ga, dW, red, crank);
+    ns_backward_tail_dev<TC, CL>(m, Wr, hdr, Ga, dW, red, crank);
     return;
   }
   if (T == 0)
@@ -1710,27 +1726,23 @@ __device__ void ns_backward_dev(int m, int T, const float* Wr, const float* Xh, 
     if (CL > 1) phase_sync<CL>();
     G = Gn; Gn = Gn == Ga ? Gb : Ga;
   }
-  ns_backward_tail_dev<CL>(m, Wr, hdr, G, dW, red, crank);
+  ns_backward_tail_dev<TC, CL>(m, Wr, hdr, G, dW, red, crank);
 }
 
 // End of the adjoint: X_0 = alpha Wr^T with alpha = 1 / (||Wr||_1 ||Wr||_inf) (unless given).  G = dLoss/dX_0 and dW
 // (the part accumulated over the steps) are fp32 [m][m] in global memory; dW receives the rest.  CL CTAs share it.
-// SYM: Wr is symmetric bit for bit (the landmark kernel matrix is), so <G, Wr^T> is read along the rows of both.
-template <int CL, bool SYM>
+template <bool TC, int CL>
 __device__ void ns_backward_tail_dev(int m, const float* Wr, const NsHdr* hdr, const float* G, float* dW, float* red, int crank) {
   const int tid = threadIdx.x, gt = crank * 256 + tid, gn = 256 * CL;
   const long long mm = (long long)m * m;
   const float alpha = hdr->alpha;
   float part = 0.f;
-  if (SYM) {
-    float p4[4] = {0.f, 0.f, 0.f, 0.f};              // four independent chains: the loads of a batch overlap
-    long long e = tid;
-    for (; e + 3 * 256 < mm; e += 4 * 256) {
-#pragma unroll
-      for (int u = 0; u < 4; ++u) p4[u] += G[e + u * 256] * Wr[e + u * 256];
+  if (TC) {                                          // every CTA of a cluster sums everything, one chain per thread
+#pragma unroll 4
+    for (unsigned e = (unsigned)tid; e < (unsigned)mm; e += 256u) {
+      const unsigned i = e / (unsigned)m, j = e - i * (unsigned)m;
+      part += G[e] * Wr[j * (unsigned)m + i];
     }
-    for (; e < mm; e += 256) p4[0] += G[e] * Wr[e];
-    part = (p4[0] + p4[1]) + (p4[2] + p4[3]);
   } else {
     float p4[4] = {0.f, 0.f, 0.f, 0.f};              // a share of the sum per CTA of the cluster
     const unsigned um = (unsigned)m, umm = um * um;
@@ -1744,7 +1756,7 @@ __device__ void ns_backward_tail_dev(int m, const float* Wr, const NsHdr* hdr, c
     part = (p4[0] + p4[1]) + (p4[2] + p4[3]);
   }
   float dalpha = block_sum(part, red);
-  if constexpr (CL > 1 && !SYM) dalpha = cluster_sum<CL>(dalpha, red + 64, crank);
+  if constexpr (CL > 1 && !TC) dalpha = cluster_sum<CL>(dalpha, red + 64, crank);
 #pragma unroll 4
   for (unsigned e = (unsigned)gt; e < (unsigned)mm; e += (unsigned)gn) {      // dW[j][i] += alpha G[i][j]
     const unsigned j = e / (unsigned)m, i = e - j * (unsigned)m;

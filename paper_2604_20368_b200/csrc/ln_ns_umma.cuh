@@ -171,17 +171,15 @@ __device__ bool ns_forward_umma(int m, int T, float eps, float alpha_in, const f
   __syncthreads();
   {
     float* colsum = red; float* rowsum = red + 256;
-    {   // the first 128 threads take the columns, the others the rows (rotated start: no bank conflicts; padding is zero);
-        // four sums per thread keep the additions of a thread apart
+    {   // the first 128 threads take the columns, the others the rows (rotated start: no bank conflicts; padding is zero).
+        // One chain of additions per sum, in this order: the scale of X_0, and with it the bits of every output, hangs on it.
       const int t = tid & 127;
       if (t < UM) {
-        float c4[4] = {0.f, 0.f, 0.f, 0.f};
         const bool cols = tid < 128;
-#pragma unroll 4
-        for (int i = 0; i < UM; i += 4)
-#pragma unroll
-          for (int u = 0; u < 4; ++u) c4[u] += fabsf(Wf[cols ? (i + u) * UM + t : t * UM + ((i + u + t) & (UM - 1))]);
-        (cols ? colsum : rowsum)[t] = (c4[0] + c4[1]) + (c4[2] + c4[3]);
+        float sum = 0.f;
+#pragma unroll 8
+        for (int i = 0; i < UM; ++i) sum += fabsf(Wf[cols ? i * UM + t : t * UM + ((i + t) & (UM - 1))]);
+        (cols ? colsum : rowsum)[t] = sum;
       }
     }
     __syncthreads();

@@ -286,6 +286,35 @@ def test_fp32_newton_schulz_variants_at_their_edges(m):
         assert rel_err(f64(dW), dWo) < 1e-4
 
 
+@pytest.mark.parametrize("lm_mode,mh,mw", [(1, 3, 4), (1, 7, 7), (1, 8, 8), (1, 5, 13), (1, 8, 16),
+                                           (3, 7, 7), (3, 8, 8), (3, 8, 12), (3, 8, 16), (3, 14, 14)])
+def test_bf16_scale_of_x0_is_formed_from_sums_in_one_order(lm_mode, mh, mw):
+    """Without an iteration X = X_0 = alpha W^T, alpha = 1 / (||W||_1 ||W||_inf).  The norms are fp32 sums in a fixed order:
+    columns from the top; rows from the left (two landmark sets) or from the diagonal on, around the padded width (one
+    set).  Another order moves alpha by a unit in the last place and with it the rounding of the bf16 outputs."""
+    gh, gw, d, H, m = 28, 32, 64, 4, mh * mw
+    gen = torch.Generator().manual_seed(77 + m)
+    Q, K, V = (torch.randn(2, H, gh * gw, d, generator=gen).to(torch.bfloat16).to(DEV) for _ in range(3))
+    eps = np.float32(1e-3)
+    p = ln.Problem(2, H, gh * gw, d, m, float(d), 0, ridge_eps=float(eps), lm_mode=lm_mode, gh=gh, gw=gw, mh=mh, mw=mw)
+    saved = torch.empty(ln.laplace_nystrom_saved_bytes(p), dtype=torch.uint8, device=DEV)
+    ln.laplace_nystrom_fwd(p, Q, K, V, saved=saved)
+    W = ln.binding.saved_array(p, saved, "W").cpu().numpy()
+    X = ln.binding.saved_array(p, saved, "X").cpu().numpy()
+    Wr = W + eps * np.eye(m, dtype=np.float32)
+    wide = m if lm_mode == 3 else (64 if m <= 64 else 128)
+    A = np.zeros((Wr.shape[0], wide, wide), np.float32)
+    A[:, :m, :m] = np.abs(Wr)
+    t = np.arange(wide)
+    cols, rows = np.zeros(A.shape[:2], np.float32), np.zeros(A.shape[:2], np.float32)
+    for i in range(wide):
+        cols += A[:, i, :]
+        rows += A[:, t, i if lm_mode == 3 else (i + t) % wide]
+    alpha = np.float32(1) / (cols.max(1) * rows.max(1))
+    assert alpha.dtype == np.float32
+    np.testing.assert_array_equal(X, alpha[:, None, None] * Wr.transpose(0, 2, 1))
+
+
 @pytest.mark.parametrize("mh,mw", [(5, 6), (7, 8), (8, 8), (5, 13), (10, 13)])
 def test_fp32_storage_path_over_the_solver_variants(mh, mw):
     cfg = synth.Config("f32_edges", B=1, H=2, d=64, m=mh * mw, T=4, gh=20, gw=20, mh=mh, mw=mw, prefix=1,
