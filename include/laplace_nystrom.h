@@ -202,6 +202,7 @@ int ns_pinv(int32_t batch, int32_t m, const float* W, int32_t iters, float ridge
  * Adjoint of ns_pinv: given dX = dLoss/dX_T returns dW = dLoss/dW [batch,m,m] (W before the ridge).
  * X_hist: the [batch,iters+1,m,m] history a previous ns_pinv wrote, or NULL to recompute it.
  * With alpha <= 0 the dependence of alpha on W is differentiated (arg-max ties -> lowest index).
+ * dW may be the buffer of dX itself (in place); any other overlap of the two is not supported.
  * ws: ns_pinv_workspace_bytes(batch, m, iters).
  */
 int ns_pinv_bwd(int32_t batch, int32_t m, const float* W, int32_t iters, float ridge_eps, float alpha,

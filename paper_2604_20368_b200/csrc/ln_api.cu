@@ -1247,6 +1247,10 @@ int ns_pinv_bwd(int32_t batch, int32_t m, const float* W, int32_t iters, float r
   {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int cl = ns_cluster(m);
+    if (dX == dW && cl > 1) {        // in place: the kernel writes dW in phases that still read dX (one CTA reads it all first)
+      if (cudaMemcpyAsync(w.Gb, dX, (size_t)batch * m * m * sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess) return LN_ERR_CUDA;
+      dX = w.Gb;
+    }
     auto go = [&](auto kern) {
       const size_t smem = cl == 1 ? kResBwdSmem : sizeof(GemmSmem);
       want_smem(kern, smem);

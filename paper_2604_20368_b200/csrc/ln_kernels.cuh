@@ -1684,7 +1684,8 @@ __device__ void ns_backward_tail_dev(int m, const float* Wr, const NsHdr* hdr, c
 
 // =====================================================================================
 // Exact adjoint of ns_forward_dev: given G0 = dLoss/dX_T returns dW = dLoss/dW.
-// Scratch matrices [m][m]: P, Hm, Ga, Gb.  Xh holds X_0..X_T, Wr = W + eps I, hdr from the forward.
+// Scratch matrices [m][m]: P, Hm, Ga, Gb.  Xh holds X_0..X_T, Wr = W + eps I, hdr from the forward.  G0 may be Gb; it must
+// not be dW, which is written while G0 is still read (m <= 64 excepted).
 // =====================================================================================
 template <bool TC, int CL = 1>
 __device__ void ns_backward_dev(int m, int T, const float* Wr, const float* Xh, const NsHdr* hdr,

@@ -286,6 +286,23 @@ def test_fp32_newton_schulz_variants_at_their_edges(m):
         assert rel_err(f64(dW), dWo) < 1e-4
 
 
+@pytest.mark.parametrize("m", [16, 49, 64, 65, 128, 200])
+@pytest.mark.parametrize("T", [0, 3])
+def test_ns_pinv_bwd_in_place(m, T):
+    """dW may be the buffer that holds dX: the same bits as with a buffer of its own, with and without the history."""
+    lib, ptr = ln.binding.lib(), ln.binding._ptr
+    W = torch.from_numpy(_kernel_matrices(3, m, 16, 5 + m).astype(np.float32)).to(DEV)
+    dX = torch.from_numpy(np.random.default_rng(m).standard_normal(W.shape).astype(np.float32)).to(DEV)
+    _, hist, _ = ln.ns_pinv(W, T, ridge_eps=1e-6, want_hist=True)
+    ws = torch.empty(lib.ns_pinv_workspace_bytes(3, m, T), dtype=torch.uint8, device=DEV)
+    for h in (None, hist):
+        ref = ln.ns_pinv_bwd(W, T, 1e-6, 0.0, dX, X_hist=h)
+        buf = dX.clone()
+        assert lib.ns_pinv_bwd(3, m, ptr(W), T, 1e-6, 0.0, ptr(h), ptr(buf), ptr(buf), ptr(ws), ws.numel(),
+                               ln.binding._stream()) == 0
+        assert torch.equal(buf, ref)
+
+
 @pytest.mark.parametrize("lm_mode,mh,mw", [(1, 3, 4), (1, 7, 7), (1, 8, 8), (1, 5, 13), (1, 8, 16),
                                            (3, 7, 7), (3, 8, 8), (3, 8, 12), (3, 8, 16), (3, 14, 14)])
 def test_bf16_scale_of_x0_is_formed_from_sums_in_one_order(lm_mode, mh, mw):
