@@ -1590,21 +1590,34 @@ __device__ void ns_forward_dev(int m, int T, float eps, float alpha_in, const fl
   // both norms, every CTA of a cluster for itself
   float* colsum = red;          // [256]
   float* rowsum = red + 256;    // [256]
-  for (unsigned e = (unsigned)gt; e < umm; e += (unsigned)gn) Wr[e] = W[e] + (e % (um + 1u) == 0u ? eps : 0.f);
   if constexpr (TC) {
     // One chain of additions per sum, in index order: the scale of X_0, and with it the bits of every bf16 output, hangs
-    // on it.  Up to 128 columns half of the threads take the rows beside the other half's columns.
+    // on it.  Up to 128 columns half of the threads take the rows beside the other half's columns.  A row's values come
+    // four at a time where they can: 32 lanes read 32 rows, one line each.
     const int mp = m <= 128 ? 128 : 256;
     for (int s = tid; s < 2 * mp; s += 256) {
       const bool cols = s < mp;
       const int t = cols ? s : s - mp;
+      if (t >= m) continue;
+      const float* const p = W + (cols ? t : t * m);
       float sum = 0.f;
-      if (t < m) {
+      if (cols) {
+#pragma unroll 16
+        for (int i = 0; i < m; ++i) sum += fabsf(p[i * m] + (i == t ? eps : 0.f));
+      } else if ((m & 3) == 0) {
+#pragma unroll 4
+        for (int i = 0; i < m; i += 4) {
+          const float4 w = ld4(p + i);
+          sum += fabsf(w.x + (i == t ? eps : 0.f));     sum += fabsf(w.y + (i + 1 == t ? eps : 0.f));
+          sum += fabsf(w.z + (i + 2 == t ? eps : 0.f)); sum += fabsf(w.w + (i + 3 == t ? eps : 0.f));
+        }
+      } else {
 #pragma unroll 8
-        for (int i = 0; i < m; ++i) sum += fabsf(W[cols ? i * m + t : t * m + i] + (i == t ? eps : 0.f));
-        (cols ? colsum : rowsum)[t] = sum;
+        for (int i = 0; i < m; ++i) sum += fabsf(p[i] + (i == t ? eps : 0.f));
       }
+      (cols ? colsum : rowsum)[t] = sum;
     }
+    for (unsigned e = (unsigned)gt; e < umm; e += (unsigned)gn) Wr[e] = W[e] + (e % (um + 1u) == 0u ? eps : 0.f);
   } else {
     // one pass over W: a warp takes every eighth row, a lane every 32nd column; four rows are in flight together
     float* colpart = reinterpret_cast<float*>(&sm);      // [8][256]
@@ -1638,6 +1651,7 @@ __device__ void ns_forward_dev(int m, int T, float eps, float alpha_in, const fl
 #pragma unroll
       for (int v = 0; v < 8; ++v) colpart[warp * 256 + lane + 32 * v] = cs[v];
     }
+    for (unsigned e = (unsigned)gt; e < umm; e += (unsigned)gn) Wr[e] = W[e] + (e % (um + 1u) == 0u ? eps : 0.f);
     __syncthreads();
     if (tid < m) {
       float t = 0.f;
