@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(256, 3) k_nn_umma(const float* __restrict__ E,
       *reinterpret_cast<uint4*>(O + (long long)i * D + c8) = make_uint4(wo[0], wo[1], wo[2], wo[3]);
     }
     if (warp == 0) umma::tmem_dealloc(tmem_base, D);
-    if (!ok && dev_status && tid == 0) atomicOr(dev_status + bh, 2);
+    umma::report_timeout(ok, dev_status, bh);
     return;
   }
   {
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(256, 3) k_nn_umma(const float* __restrict__ E,
     if (i0 + r < n) *reinterpret_cast<uint4*>(O + (long long)(i0 + r) * D + c8) = *reinterpret_cast<const uint4*>(stage + r * LDS_ + c8);
   }
   if (warp == 0) umma::tmem_dealloc(tmem_base, D);
-  if (!ok && dev_status && tid == 0) atomicOr(dev_status + bh, 2);
+  umma::report_timeout(ok, dev_status, bh);
 }
 
 // =====================================================================================
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(256, 2) k_ntg_umma(const bf16* __restrict__ U,
   umma::fence_before_sync();
   __syncthreads();
   if (warp == 0) umma::tmem_dealloc(tmem_base, ncols);
-  if (!ok && dev_status && tid == 0) atomicOr(dev_status + bh, 2);
+  umma::report_timeout(ok, dev_status, bh);
 }
 
 }  // namespace ln

@@ -2172,7 +2172,8 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
     if constexpr (MP == 0)
       for (int e = tid; e < m * m; e += 256) bad += isfinite(XT[(long long)(e / m) * ldx + e % m]) ? 0.f : 1.f;
     bad = block_sum(bad, red);
-    if (tid == 0 && crank == 0) atomicOr(dev_status + bh, (bad > 0.f ? 1 : 0) | (tc_ok ? 0 : 2));   // bit1: a bounded tensor-core wait ran out
+    if (tid == 0 && crank == 0 && bad > 0.f) atomicOr(dev_status + bh, 1);
+    umma::report_timeout(tc_ok, dev_status, bh);
   }
   }
   if (!(phase & 2)) return;
@@ -2192,7 +2193,7 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
     if (!(phase & 1)) u2_begin(u2c, ctl256, mbars256, reinterpret_cast<bf16*>(dyn_smem), 256);
     const bool y_ok = u2_product_y(u2c, m, D, Wr, Mout, P, Y, crank);
     umma_end(ctl256, 256);
-    if (dev_status && !y_ok && tid == 0 && crank == 0) atomicOr(dev_status + bh, 2);
+    umma::report_timeout(y_ok, dev_status, bh);
     phase_sync<CL>();
   } else {
     ns_gemm<TC, false, false>(m, D, m, XT, ldx, Mout, D, Y, D, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);   // Y = X M
@@ -2332,7 +2333,7 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
     u2_begin(u2c, ctl256, mbars256, reinterpret_cast<bf16*>(dyn_smem), 512);
     const bool p_ok = u2_products_dx_dm(u2c, m, D, dY, Msaved, XT, Hm, Gb, dXm, dM, crank);
     if (!(phase & 2)) umma_end(ctl256, 512);
-    if (dev_status && !p_ok && tid == 0 && crank == 0) atomicOr(dev_status + bh, 2);
+    umma::report_timeout(p_ok, dev_status, bh);
   } else {
     ns_gemm<TC, false, true>(m, m, D, dY, D, Msaved, D, dXm, ldx, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);   // dX = dY M^T
     ns_gemm<TC, true, false>(m, D, m, XT, ldx, dY, D, dM, D, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);        // dM = X^T dY
@@ -2347,12 +2348,12 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
   if constexpr (MP == 128 || MP == 64) {
     __shared__ UmmaCtl ctl;
     const bool tc_ok = ns_backward_umma<MP>(m, T, eps, W, Xh, Ph, ldx, mx, hdr, dXm, GW, ldm, inv_lambda, reinterpret_cast<bf16*>(dyn_smem), red, ctl);
-    if (dev_status && !tc_ok && tid == 0) atomicOr(dev_status + bh, 2);
+    umma::report_timeout(tc_ok, dev_status, bh);
   } else if constexpr (MP == 256) {
     if (!(phase & 1)) u2_begin(u2c, ctl256, mbars256, reinterpret_cast<bf16*>(dyn_smem), 512);
     const bool tc_ok = ns_backward_umma256(u2c, m, T, Xh, Ph, dXm, Ga, Gb, Hm, Wr, P, dWm, crank);
     umma_end(ctl256, 512);
-    if (dev_status && !tc_ok && tid == 0 && crank == 0) atomicOr(dev_status + bh, 2);
+    umma::report_timeout(tc_ok, dev_status, bh);
     // end of the adjoint and GW in one pass (the operand buffers are free: the engine has ended with a cluster barrier)
     ns_tail_gw_sym<CL>(m, ldm, W, eps, hdr, P, dWm, inv_lambda, GW, red, reinterpret_cast<float*>(dyn_smem), crank);
   } else if (solver == 0) { ns_backward_dev<TC, CL>(m, T, Wr, Xh, hdr, dXm, dWm, P, Hm, Ga, Gb, sm, red, crank, Ph); if (CL > 1) phase_sync<CL>(); }
@@ -2377,17 +2378,16 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
 // =====================================================================================
 // Self-test of the bounded wait every tensor-core kernel of this library uses: an mbarrier on which nothing ever
 // arrives is waited for with a probe limit; the wait must give up, and the kernel reports it the way the product
-// kernels do (bit 1 of the status word) and returns normally.
+// kernels do (bit 1 of the status word, by the thread that waited: here the last lane) and returns normally.
 // =====================================================================================
 __global__ void k_selftest_wait(int probes, int* dev_status) {
   pdl_wait();
   __shared__ __align__(8) unsigned long long mbar;
   if (threadIdx.x == 0) umma::mbar_init(&mbar, 1);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const bool ok = umma::mbar_wait(&mbar, 0, probes);
-    if (!ok) atomicOr(dev_status, 2);
-  }
+  bool ok = true;
+  if (threadIdx.x == 31) ok = umma::mbar_wait(&mbar, 0, probes);
+  umma::report_timeout(ok, dev_status, 0);
 }
 
 // =====================================================================================

@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(256, 2) k_sign3(const bf16* __restrict__ tok, 
     umma::fence_before_sync();
     __syncthreads();
     if (warp == 0) umma::tmem_dealloc(tmem_base, ncols);
-    if (!ok && dev_status && tid == 0) atomicOr(dev_status + bh, 2);
+    umma::report_timeout(ok, dev_status, bh);
   }
 }
 

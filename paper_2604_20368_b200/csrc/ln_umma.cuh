@@ -84,6 +84,11 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* mbar, uint32_t par
                  : "=r"(done) : "r"(s32(mbar)), "r"(parity) : "memory");
   return done != 0;
 }
+// A wait that ran out is reported by the thread that waited: where one thread issues, that is the lane elect.sync gives,
+// which need not be lane 0.
+__device__ __forceinline__ void report_timeout(bool ok, int* dev_status, int head) {
+  if (!ok && dev_status) atomicOr(dev_status + head, 2);
+}
 
 // Bulk copy global -> shared of `bytes` (a multiple of 16, both addresses 16-byte aligned) by ONE thread; the
 // bytes are counted on `mbar`, which must have been told to expect them (expect_tx) beforehand.

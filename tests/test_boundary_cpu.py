@@ -224,3 +224,17 @@ def test_saved_array_views_lie_inside_the_context(name):
     for (a0, a1, na), (b0, b1, nb) in zip(spans, spans[1:]):
         assert a1 <= b0 or {na, nb} == {"X"}, (na, nb)
     assert binding.lib().laplace_nystrom_saved_array(ctypes.byref(cp), b"nope", info) == -1
+
+
+def test_a_wait_that_ran_out_is_reported_by_the_thread_that_waited():
+    """Bulk copies and tensor-core work are issued, and often waited for, by the one lane elect.sync gives, which need not
+    be thread 0: the kernels hand the outcome of a bounded wait to report_timeout on every thread, with no test of the
+    thread index in front of bit 1 of the status word."""
+    csrc = os.path.join(ROOT, "paper_2604_20368_b200", "csrc")
+    reported = 0
+    for name in sorted(os.listdir(csrc)):
+        for line in open(os.path.join(csrc, name)):
+            if re.search(r"!\s*\w*ok\b.*atomicOr|atomicOr.*\bok\b.*2\)", line):
+                assert not re.search(r"\btid\b|threadIdx|crank", line), (name, line)
+            reported += "umma::report_timeout(" in line
+    assert reported >= 10          # product kernels (4), per-head kernels (5), self-test (1)
