@@ -462,12 +462,21 @@ void launch_clustered(void (*kern)(KArgs...), int grid, int cl, size_t smem, cud
   cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
 
-// landmark pooling: one thread per (landmark, 4 channels) for small bins, a CTA per landmark for large ones
+// Landmark pooling: one thread per (landmark, 4 channels) for small bins, a CTA per landmark for large ones.
+// Small bins: with eight tokens of a bin in flight a thread waits less, but the 62 (bf16) or 78 (fp32) registers leave four
+// or three CTAs per SM instead of five.  That pays where the whole grid is resident at two CTAs per SM (bins of 9 to 63
+// tokens 0.75 to 1.0 of the time in fp32, 0.8 to 1.0 in bf16, 3 x 4 bins there 1.05), and with long bins in fp32 on grids of
+// several waves (7 x 7 on 768 CTAs 0.66, on 2304 CTAs 0.92, but 1.15 on 512, one wave at five per SM); many CTAs with short bins keep memory busy by themselves and lose (3 x 4 on 2688 CTAs 1.13 to 1.16, 4 x 4
+// on 512 CTAs 1.17 in fp32; bf16 at 36 tokens on 512 to 6912 CTAs 0.97 to 1.14).  Up to eight tokens: never.
 template <typename T>
 void launch_pool(const ln_problem* p, const T* src, float* L, cudaStream_t st) {
   const int bin_tokens = ((p->gh + p->mh - 1) / p->mh) * ((p->gw + p->mw - 1) / p->mw);
-  if (bin_tokens >= 64) LN_LAUNCH("k_pool", st, enqueue(k_pool_wide<T>, dim3(p->m, p->B * p->H), 256, 0, st, src, L, geom_of(p)));
-  else LN_LAUNCH("k_pool", st, enqueue(k_pool<T>, dim3(cdiv(p->m, 256 / (p->d / 4)), p->B * p->H), 256, 0, st, src, L, geom_of(p)));
+  const int BH = p->B * p->H, per_head = cdiv(p->m, 256 / (p->d / 4));
+  const long long ctas = (long long)per_head * BH, sms = sm_count();
+  if (bin_tokens >= 64) LN_LAUNCH("k_pool", st, enqueue(k_pool_wide<T>, dim3(p->m, BH), 256, 0, st, src, L, geom_of(p)));
+  else if (bin_tokens > 8 && (ctas <= 2 * sms || (std::is_same<T, float>::value && bin_tokens >= 49 && ctas > 4 * sms)))
+    LN_LAUNCH("k_pool", st, enqueue(k_pool<T, true>, dim3(per_head, BH), 256, 0, st, src, L, geom_of(p)));
+  else LN_LAUNCH("k_pool", st, enqueue(k_pool<T, false>, dim3(per_head, BH), 256, 0, st, src, L, geom_of(p)));
 }
 
 template <typename T> constexpr int is_f32() { return std::is_same<T, float>::value ? 1 : 0; }

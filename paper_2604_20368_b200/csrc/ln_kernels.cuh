@@ -369,8 +369,6 @@ template <typename T> __global__ void k_to_f32(const T* __restrict__ x, float* _
 // =====================================================================================
 // Landmark selection: adaptive average pooling of the keys over the token grid (Sec. 4.2)
 // =====================================================================================
-// filt: NULL = average pooling; else the depth-wise-convolution selection of Sec. 4.2, one filter per head and channel,
-// [H][taps][d] with taps = (gh/mh) * (gw/mw) (the grid divides: the host checks), tap (u, v) of a region at u (gw/mw) + v
 // four consecutive elements as they lie in memory, and as fp32
 template <typename T> struct Raw4;
 template <> struct Raw4<float> {
@@ -383,14 +381,17 @@ template <> struct Raw4<bf16> {
     return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16), __uint_as_float(r.y & 0xffff0000u));
   }
 };
+// filt: NULL = average pooling; else the depth-wise-convolution selection of Sec. 4.2, one filter per head and channel,
+// [H][taps][d] with taps = (gh/mh) * (gw/mw) (the grid divides: the host checks), tap (u, v) of a region at u (gw/mw) + v
 struct PoolGeom { int n, d, m, prefix, gh, gw, mh, mw; const float* filt; int H; };
 // 32-bit on purpose (64-bit division costs two orders of magnitude more on the device); the host
 // checks that gh * mh and gw * mw stay below 2^31.
 __host__ __device__ inline int bin_lo(int a, int g, int mb) { return (int)(((unsigned)a * (unsigned)g) / (unsigned)mb); }
 __host__ __device__ inline int bin_hi(int a, int g, int mb) { return (int)(((unsigned)(a + 1) * (unsigned)g + (unsigned)mb - 1u) / (unsigned)mb); }
 
-// grid (ceil(m / (256 / (d/4))), BH); thread = (landmark, 4 dims)
-template <typename T>
+// grid (ceil(m / (256 / (d/4))), BH); thread = (landmark, 4 dims).  BATCH: eight tokens of the bin in flight, added in their
+// order (7 x 7-token bins at 32 heads x 3136 tokens, bf16, 64 dims 23.7 -> 17.3 us; launch_pool chooses).
+template <typename T, bool BATCH>
 __global__ void __launch_bounds__(256) k_pool(const T* __restrict__ K, float* __restrict__ L, PoolGeom g) {
   pdl_wait();
   const int quads = g.d / 4, lpb = 256 / quads;
@@ -411,15 +412,9 @@ __global__ void __launch_bounds__(256) k_pool(const T* __restrict__ K, float* __
       s0 += (double)w.x * (double)f.x; s1 += (double)w.y * (double)f.y; s2 += (double)w.z * (double)f.z; s3 += (double)w.w * (double)f.w;
     } else { s0 += (double)f.x; s1 += (double)f.y; s2 += (double)f.z; s3 += (double)f.w; }
   };
-  const int ntok = (r1 - r0) * (c1 - c0);
-  const T* row = Kh + (long long)(g.prefix + r0 * g.gw) * g.d + c;
-  if (ntok <= 8) {
-    for (int t = 0, r = r0; r < r1; ++r, row += (long long)g.gw * g.d)
-      for (int q = c0; q < c1; ++q, ++t) add(ld4(row + (long long)q * g.d), t);
-  } else {
-    // Eight tokens of the bin in flight, added in their order: with 7 x 7-token bins at 32 heads x 3136 tokens 23.7 ->
-    // 17.3 us, with 4 x 4 in fp32 at 32 heads x 784 13.8 -> 9.2 us.  Up to eight tokens the loads are too few for the
-    // bookkeeping to pay (2 x 2 bins at 384 heads x 197: 14.1 against 16.6 us).
+  if constexpr (BATCH) {
+    const int ntok = (r1 - r0) * (c1 - c0);
+    const T* row = Kh + (long long)(g.prefix + r0 * g.gw) * g.d + c;
     for (int t0 = 0, q = c0; t0 < ntok; t0 += 8) {
       typename Raw4<T>::type v[8];
 #pragma unroll
@@ -433,6 +428,9 @@ __global__ void __launch_bounds__(256) k_pool(const T* __restrict__ K, float* __
         add(Raw4<T>::f(v[u]), t0 + u);
       }
     }
+  } else {
+    for (int r = r0; r < r1; ++r)
+      for (int q = c0; q < c1; ++q) add(ld4(Kh + (long long)(g.prefix + r * g.gw + q) * g.d + c), (r - r0) * (c1 - c0) + (q - c0));
   }
   const double cnt = wf ? 1.0 : (double)((r1 - r0) * (c1 - c0));
   st4(L + ((long long)bh * g.m + l) * g.d + c,

@@ -93,18 +93,21 @@ def test_l1_kernel_bwd(batch, na, nb, d, dtype, recompute):
     assert rel_err(f64(dB), dBo) < tol
 
 
-@pytest.mark.parametrize("gh,gw,mh,mw,prefix", [(8, 8, 4, 4, 0), (9, 8, 3, 4, 1), (12, 9, 4, 3, 1), (16, 16, 4, 4, 0),
-                                                (29, 21, 4, 3, 1), (7, 63, 1, 1, 0)])
+@pytest.mark.parametrize("gh,gw,mh,mw,prefix", [(8, 8, 4, 4, 0), (9, 8, 3, 4, 1), (8, 16, 4, 4, 1), (12, 9, 4, 3, 1),
+                                                (16, 16, 4, 4, 0), (29, 21, 4, 3, 1), (16, 16, 2, 2, 0), (7, 63, 1, 1, 0)])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
-def test_landmarks_pool_bin_sizes(gh, gw, mh, mw, prefix, dtype):
-    """Bins of 4, 6 to 9, 9, 16, 56 to 64 (overlapping) and 441 tokens: below, at and above the eight tokens from which
-    the loads are batched, and the kernel for large bins.  A landmark is the fp32 value nearest to the exact mean."""
+@pytest.mark.parametrize("B", [2, 100])
+def test_landmarks_pool_bin_sizes(gh, gw, mh, mw, prefix, dtype, B):
+    """Bins of 4, 6, 8, 9, 16, 56 (overlapping rows), 64 and 441 tokens: up to the eight tokens that are read one by one,
+    above them, and the kernel for large bins from 64 tokens on; few heads, where a bin of nine tokens or more is read eight
+    at a time, and many, where only the long bins of fp32 storage are.  A landmark is the fp32 value nearest to the exact
+    mean."""
     n, d = prefix + gh * gw, 64
-    K = _rand((2, 3, n, d), 31, dtype)
-    p = ln.problem_from_config(synth.Config("bins", B=2, H=3, d=d, m=mh * mw, T=1, gh=gh, gw=gw, mh=mh, mw=mw, prefix=prefix,
+    K = _rand((B, 3, n, d), 31, dtype)
+    p = ln.problem_from_config(synth.Config("bins", B=B, H=3, d=d, m=mh * mw, T=1, gh=gh, gw=gw, mh=mh, mw=mw, prefix=prefix,
                                             dtype="f32" if dtype == torch.float32 else "bf16", seed=1), whiten=None)
     L = ln.landmarks_pool(p, K.to(DEV))
-    G = f64(K)[:, :, prefix:].reshape(2, 3, gh, gw, d)
+    G = f64(K)[:, :, prefix:].reshape(B, 3, gh, gw, d)
     lo, hi = lambda a, g, m: a * g // m, lambda a, g, m: -(-(a + 1) * g // m)
     ref = np.stack([G[:, :, lo(a, gh, mh):hi(a, gh, mh), lo(b, gw, mw):hi(b, gw, mw)].mean(axis=(2, 3))
                     for a in range(mh) for b in range(mw)], axis=2)
