@@ -933,17 +933,27 @@ NsWs carve_ns_ws(int batch, int m, int T, void* base) {
 }
 
 // CTAs of a thread-block cluster that share one matrix of the stand-alone Newton-Schulz entry points (the output tiles of
-// every product are dealt out to them); up to 64 the matrices of a step fit one CTA's shared memory
-int ns_cluster(int m) { return m > 64 ? 8 : 1; }
+// every product are dealt out to them).  Up to 64 landmarks the matrices of a step fit one CTA's shared memory, with one
+// CTA per SM; at every batch that beats two CTAs per SM on matrices in L2 (T = 6, forward / adjoint, 16 x 16, 49 x 49 and
+// 64 x 64: batch 64 17 / 45 -> 9 / 18, 66 / 149 -> 30 / 64, 74 / 163 -> 35 / 89 us; batch 512 47 / 121 -> 34 / 71,
+// 165 / 404 -> 114 / 250, 191 / 491 -> 139 / 359).  Beyond, eight CTAs give the shortest chain while every cluster is
+// resident at two CTAs per SM.  A cluster stays within one part of the chip, so nine tenths of the places can be had (33
+// matrices on 148 SMs: forward / adjoint 76 / 165 us at 65 landmarks, 99 / 211 at 128; with 34 131 / 269 and 162 / 339).
+// With more matrices than that four CTAs, which repeat less of the work: batch 34 110 / 250 and 153 / 329, batch 64
+// 113 / 254 and 158 / 347 (eight CTAs 152 / 332 and 197 / 425).  More than 128 landmarks have sixteen or more tiles: eight.
+int ns_cluster(int m, int batch) {
+  if (m <= 64) return 1;
+  return m > 128 || 80ll * batch <= 18ll * sm_count() ? 8 : 4;
+}
 void launch_ns_pinv(int batch, int m, int iters, float eps, float alpha, const float* W, const NsWs& w, float* Xh, float* X,
                     float* resid, cudaStream_t st) {
-  const int cl = ns_cluster(m);
+  const int cl = ns_cluster(m, batch);
   auto go = [&](auto kern) {
     const size_t smem = cl == 1 ? kResFwdSmem : sizeof(GemmSmem);
     want_smem(kern, smem);
     LN_LAUNCH("k_ns_pinv", st, launch_clustered(kern, batch * cl, cl, smem, st, m, iters, eps, alpha, W, w.Wr, w.P, Xh, w.hdr, X, resid));
   };
-  if (cl == 8) go(k_ns_pinv<8>); else go(k_ns_pinv<1>);
+  if (cl == 8) go(k_ns_pinv<8>); else if (cl == 4) go(k_ns_pinv<4>); else go(k_ns_pinv<1>);
 }
 }  // namespace
 
@@ -1255,7 +1265,7 @@ int ns_pinv_bwd(int32_t batch, int32_t m, const float* W, int32_t iters, float r
   const NsWs w = carve_ns_ws(batch, m, iters, ws);
   {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int cl = ns_cluster(m);
+    const int cl = ns_cluster(m, batch);
     if (dX == dW && cl > 1) {        // in place: the kernel writes dW in phases that still read dX (one CTA reads it all first)
       if (cudaMemcpyAsync(w.Gb, dX, (size_t)batch * m * m * sizeof(float), cudaMemcpyDeviceToDevice, st) != cudaSuccess) return LN_ERR_CUDA;
       dX = w.Gb;
@@ -1266,7 +1276,7 @@ int ns_pinv_bwd(int32_t batch, int32_t m, const float* W, int32_t iters, float r
       LN_LAUNCH("k_ns_pinv_bwd", st, launch_clustered(kern, batch * cl, cl, smem, st, m, iters, ridge_eps, alpha, W, w.Wr, w.P, w.Hm, w.Ga, w.Gb, w.Xh,
                                                       X_hist, w.hdr, dX, dW));
     };
-    if (cl == 8) go(k_ns_pinv_bwd<8>); else go(k_ns_pinv_bwd<1>);
+    if (cl == 8) go(k_ns_pinv_bwd<8>); else if (cl == 4) go(k_ns_pinv_bwd<4>); else go(k_ns_pinv_bwd<1>);
   }
   return launch_ok();
 }

@@ -289,6 +289,24 @@ def test_fp32_newton_schulz_variants_at_their_edges(m):
         assert rel_err(f64(dW), dWo) < 1e-4
 
 
+@pytest.mark.parametrize("m", [65, 96, 128])
+def test_ns_pinv_many_matrices_take_smaller_clusters(m):
+    """Beyond 64 landmarks a matrix is shared by eight CTAs, or by four once the batch no longer fits the GPU that way: a
+    batch of 100 gives each matrix what it has in a batch of four.  The order of a product's sums over k does not depend on
+    the split, so the iterates have the same bits; the adjoint's one scalar, <G, W^T>, is summed over the CTAs in other
+    parts, an fp32 sum of m^2 terms."""
+    W = torch.from_numpy(_kernel_matrices(4, m, 16, 9 + m)).to(DEV)
+    dX = torch.from_numpy(np.random.default_rng(m).standard_normal(W.shape).astype(np.float32)).to(DEV)
+    X, hist, _ = ln.ns_pinv(W, 5, ridge_eps=1e-6, want_hist=True)
+    dW = ln.ns_pinv_bwd(W, 5, 1e-6, 0.0, dX, X_hist=hist)
+    Wb, dXb = W.repeat(25, 1, 1), dX.repeat(25, 1, 1)
+    Xb, histb, _ = ln.ns_pinv(Wb, 5, ridge_eps=1e-6, want_hist=True)
+    assert torch.equal(Xb, X.repeat(25, 1, 1)) and torch.equal(histb, hist.repeat(25, 1, 1, 1))
+    for h in (None, histb):
+        dWb = ln.ns_pinv_bwd(Wb, 5, 1e-6, 0.0, dXb, X_hist=h)
+        assert rel_err(f64(dWb), f64(dW.repeat(25, 1, 1))) < m * 2.0 ** -24
+
+
 @pytest.mark.parametrize("m", [16, 49, 64, 65, 128, 200])
 @pytest.mark.parametrize("T", [0, 3])
 def test_ns_pinv_bwd_in_place(m, T):
