@@ -355,6 +355,13 @@ void enqueue(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStr
   cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
 }
 
+// An ordinary launch, for the kernel behind a fork to the side stream where a long per-head kernel must find its SMs free:
+// a dependent launch places its CTAs before the side stream's kernel has been released by the event.
+template <typename... KArgs, typename... Args>
+void enqueue_plain(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  kern<<<grid, block, smem, st>>>(KArgs(args)...);
+}
+
 // Side stream.  The per-head kernels (Newton-Schulz and its adjoint: one CTA or cluster per head, bound by the
 // latency of a chain of small products) do not depend on the token-sized kernels next to them, so the entry
 // points enqueue them on a second stream of the library, forked from and joined back into the caller's stream
@@ -563,11 +570,11 @@ int fwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
                 launch_clustered(kern, BH * cl, cl, smem, s, m, pl.ldm, pl.T, p->ridge_eps, p->ns_alpha, p->H, p->map_mode,
                                  whiten_eff, x.W, w.Wr, w.P, x.Xh, x.Ph, x.hdr, Mparts_src, Mparts, x.M, x.Y, x.Yt,
                                  x.ybar, dev_status, pl.hslot, umma_prod ? reinterpret_cast<bf16*>(x.Yimg) : nullptr, phase,
-                                 pl.cg ? 1 : 0, w.cg));
+                                 w.cg));
     };
-    // conjugate gradients (Sec. 5.3): fp32, one CTA per head, whatever the storage type
+    // conjugate gradients (Sec. 5.3): one CTA per head, whatever the storage type
+    if (pl.cg) { launch(k_mid_fwd<D, false, 0, 1, true>, kCgSmem); return; }
     const size_t mid_smem = TC ? sizeof(MmaGemmSmem) : (m <= 64 && kResFwdSmem > sizeof(GemmSmem) ? kResFwdSmem : sizeof(GemmSmem));
-    if (pl.cg) { launch(k_mid_fwd<D, false, 0>, sizeof(NsSmem)); return; }
     // two landmark sets (general matrix) or fp32 storage: the mma.sync or FFMA engine, shared by the CTAs of a cluster
     // beyond 64 landmarks
     if ((two || !TC) && m > 64) launch(k_mid_fwd<D, TC, 0, kMidCluster>, mid_smem, kMidCluster);
@@ -702,12 +709,17 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
   // one sign pass of a token-sized block: tokens, upstream operands (U, pre-split images of Y), kernel block A
   const bool bw = p->whiten_mode == 1;                // batch-statistic whitening: the scale is the forward pass's own estimate
   const float* const whiten_eff = bw ? p->whiten_batch : p->whiten;
+  // The conjugate-gradient kernel takes longer than a sign pass, whose CTAs fill the SMs: it is to be placed first (step of
+  // 32 heads x 400 tokens with dependent launches behind the fork -> ordinary ones: 49 landmarks, 128 dims 440 -> 355 us)
+  bool behind_cg = false;
   auto launch_sign3 = [&](const char* name, const T* tokp, const T* Up, const float* Yimgp, const float* Ap, auto* rowsp, float* partp,
                           const float* SBp, const float* kap = nullptr) {
     if constexpr (std::is_same<T, bf16>::value && (D == 64 || D == 128)) {
       auto go = [&](auto kern) {
         want_smem(kern, sign3_smem_bytes());
-        LN_LAUNCH(name, st, enqueue(kern, dim3(pl.s3_tiles, D / 64, BH), dim3(16, pl.s2_tg), sign3_smem_bytes(), st,
+        if (behind_cg) LN_LAUNCH(name, st, enqueue_plain(kern, dim3(pl.s3_tiles, D / 64, BH), dim3(16, pl.s2_tg), sign3_smem_bytes(), st,
+                      tokp, SBp, Up, reinterpret_cast<const bf16*>(Yimgp), Ap, pl.ldm, rowsp, partp, n, m, inv_lambda, dev_status, kap, p->H));
+        else LN_LAUNCH(name, st, enqueue(kern, dim3(pl.s3_tiles, D / 64, BH), dim3(16, pl.s2_tg), sign3_smem_bytes(), st,
                       tokp, SBp, Up, reinterpret_cast<const bf16*>(Yimgp), Ap, pl.ldm, rowsp, partp, n, m, inv_lambda, dev_status, kap, p->H));
       };
       using TO = std::remove_pointer_t<decltype(rowsp)>;
@@ -717,6 +729,7 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
   // The per-head kernel and the landmark-block sign pass need Z'^T dO only: with a side stream they run beside
   // the query-side kernels and are joined before the key side, which needs dM.
   const Side side = side_acquire(std::is_same<T, bf16>::value, st);
+  behind_cg = side.on() && pl.cg;
   const bool umma_prod = std::is_same<T, bf16>::value && (D == 64 || D == 128);
   auto launch_mid = [&](cudaStream_t s, int phase = 3) {
     constexpr bool TC = std::is_same<T, bf16>::value;
@@ -727,10 +740,10 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
                                                  x.W, x.Xh, x.Ph, x.hdr, x.M, w.dYtpart, w.dybpart, ch, p->ridge_eps, w.Wr, w.P,
                                                  w.Hm, w.Ga, w.Gb, w.dW, w.dX, w.dY, w.dM, w.GW, dev_status, pl.hslot,
                                                  umma_prod ? reinterpret_cast<bf16*>(w.dMimg) : nullptr, two ? 0 : 1,
-                                                 pl.cg ? 1 : 0, x.Y, w.cg, phase));
+                                                 x.Y, w.cg, phase));
     };
     const size_t mid_smem = TC ? sizeof(MmaGemmSmem) : (m <= 64 ? kResBwdSmem : sizeof(GemmSmem));
-    if (pl.cg) { launch(k_mid_bwd<D, false, 0>, sizeof(NsSmem)); return; }
+    if (pl.cg) { launch(k_mid_bwd<D, false, 0, 1, true>, kCgSmem); return; }
     if ((two || !TC) && m > 64) launch(k_mid_bwd<D, TC, 0, kMidCluster>, mid_smem, kMidCluster);
     else if (two) launch(k_mid_bwd<D, TC, 0>, mid_smem);
     else if (TC && m <= 64) launch(k_mid_bwd<D, TC, TC ? 64 : 0>, 4 * kUmmaMatBytes64);
@@ -810,7 +823,8 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
   }
   if (sign3) {
     const long long cnt = (long long)BH * m * D;
-    LN_LAUNCH("k_fold_landmarks", st, enqueue(k_fold_landmarks, cdiv(cnt / 4, 256), 256, 0, st, LfC, w.SB, D == 128 ? 5 : 4, cnt / 4));
+    if (behind_cg) LN_LAUNCH("k_fold_landmarks", st, enqueue_plain(k_fold_landmarks, cdiv(cnt / 4, 256), 256, 0, st, LfC, w.SB, D == 128 ? 5 : 4, cnt / 4));
+    else LN_LAUNCH("k_fold_landmarks", st, enqueue(k_fold_landmarks, cdiv(cnt / 4, 256), 256, 0, st, LfC, w.SB, D == 128 ? 5 : 4, cnt / 4));
     if (two) LN_LAUNCH("k_fold_landmarks", st, enqueue(k_fold_landmarks, cdiv(cnt / 4, 256), 256, 0, st, LfR, w.SBq, D == 128 ? 5 : 4, cnt / 4));
     if (qrows_f) launch_sign3("sign3_dQ_dLC", Q, dO, x.Yimg, x.C, qrows_f, w.dLCpart, w.SB, kap);
     else launch_sign3("sign3_dQ_dLC", Q, dO, x.Yimg, x.C, dQ, w.dLCpart, w.SB, kap);

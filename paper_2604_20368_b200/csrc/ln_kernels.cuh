@@ -2025,6 +2025,47 @@ __device__ void cg_dev(int m, int T, float eps, const float* W, const float* Bsr
   __syncthreads();
 }
 
+// dW = -A B^T for A, B [m][D] (the one product of the adjoint solve), fp32, k in order: 64 x 64 tiles, 16 dims per round.
+constexpr size_t kCgSmem = sizeof(double) * (64 * 17 + 16 * 72);          // the tiles of cg_matvec
+template <int D>
+__device__ void cg_dw(int m, const float* A, const float* B, float* dW, int ldw, float* sm) {
+  constexpr int P = 64 + 4;
+  static_assert(2 * 16 * P * sizeof(float) <= kCgSmem, "the operand tiles fit");
+  float* const As = sm;                                                   // [16][P]: As[kk][i]
+  float* const Bs = sm + 16 * P;
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, lr = tid >> 2, lk = (tid & 3) * 4;
+  for (int i0 = 0; i0 < m; i0 += 64)
+    for (int j0 = 0; j0 < m; j0 += 64) {
+      float acc[4][4] = {};
+      for (int k0 = 0; k0 < D; k0 += 16) {
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 a4 = i0 + lr < m ? ld4(A + (long long)(i0 + lr) * D + k0 + lk) : z;
+        const float4 b4 = j0 + lr < m ? ld4(B + (long long)(j0 + lr) * D + k0 + lk) : z;
+        __syncthreads();                                                  // the round before has been read
+        As[lk * P + lr] = a4.x; As[(lk + 1) * P + lr] = a4.y; As[(lk + 2) * P + lr] = a4.z; As[(lk + 3) * P + lr] = a4.w;
+        Bs[lk * P + lr] = b4.x; Bs[(lk + 1) * P + lr] = b4.y; Bs[(lk + 2) * P + lr] = b4.z; Bs[(lk + 3) * P + lr] = b4.w;
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < 16; ++kk) {
+          const float4 a = ld4(As + kk * P + 4 * ty), b = ld4(Bs + kk * P + 4 * tx);
+          const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[r][q] = fmaf(av[r], bv[q], acc[r][q]);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = i0 + 4 * ty + r, j = j0 + 4 * tx + q;
+          if (i < m && j < m) dW[(long long)i * ldw + j] = -acc[r][q];
+        }
+    }
+  __syncthreads();
+}
+
 // ------------------------------------------------------------------ stand-alone ns_pinv / ns_pinv_bwd
 // CL CTAs of a thread-block cluster share a matrix (grid = batch * CL): every product is split by output tiles, the
 // hardware cluster barrier ends a phase.  fp32 FFMA throughout (held to 2e-5 against the oracle).
@@ -2094,15 +2135,17 @@ __global__ void __launch_bounds__(256, CL > 1 ? 2 : 1) k_ns_pinv_bwd(int m, int 
 // MP: 0 = matrices in global memory (fp32 FFMA or the cluster-shared mma.sync engine); 64 / 128 = one CTA per head on
 // tcgen05 with the matrix padded to MP; 256 = tcgen05 on 2 x 2 blocks of 128, CL = 2 CTAs of a thread-block cluster
 // per head (grid = heads * CL).
-template <int D, bool TC, int MP, int CL = 1>
+template <int D, bool TC, int MP, int CL = 1, bool CG = false>
 __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 : 1)) k_mid_fwd(int m, int ldm, int T, float eps, float alpha_in, int H, int map_mode,
                                                  const float* __restrict__ whiten, const float* W, float* Wr,
                                                  float* P, float* Xh, float* Ph, NsHdr* hdr, const float* Mpart, int nchunks,
                                                  float* Mout, float* Y, float* Yt, float* ybar, int* dev_status,
-                                                 long long hslot, bf16* Yimg, int phase, int solver = 0, float* cgws = nullptr) {
+                                                 long long hslot, bf16* Yimg, int phase, float* cgws = nullptr) {
   pdl_wait();
-  // solver: 0 = Newton-Schulz (Alg. 2) and Y = X_T M; 1 = conjugate gradients on (W + eps I) Y = M (Sec. 5.3, Table 4;
-  // the single-CTA instantiation without tensor cores only), cgws = 4 m D doubles of scratch per head
+  // CG: conjugate gradients on (W + eps I) Y = M (Sec. 5.3, Table 4) in place of Newton-Schulz (Alg. 2) and Y = X_T M, one
+  // CTA per head, fp64; cgws = 4 m D doubles of scratch per head.  Kernels of their own, so that they keep their registers
+  // and kCgSmem bytes of shared memory whatever the fp32 engine takes: its 74 KB kept a CTA of this one from running beside
+  // the sign pass and took from the L1 cache (inference of 32 heads x 400 tokens, 128 dims, 49 landmarks 211 -> 162 us).
   // phase: bit 0 = Newton-Schulz (needs W only), bit 1 = everything that needs M (sum of the partials, Y, map fold).
   // The two halves may run as two launches, the first beside the kernels that produce M; X_T passes through
   // global memory either way.
@@ -2150,7 +2193,7 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
   __shared__ UmmaCtl ctl256;
   __shared__ __align__(8) unsigned long long mbars256[3];
   U2Ctx u2c;
-  if ((phase & 1) && solver == 0) {
+  if (!CG && (phase & 1)) {
   bool tc_ok = true;
   float bad = 0.f;                               // non-finite entries of X_T seen by this thread
   if constexpr (MP == 128 || MP == 64) {        // tcgen05 + TMEM, the matrix padded to MP x MP
@@ -2176,16 +2219,15 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
   }
   if (!(phase & 2)) return;
   if (!(phase & 1)) phase_sync<CL>();             // the M sums of all threads that share the head
-  if (solver == 1) {
-    if constexpr (!TC && MP == 0 && CL == 1) {
-      __syncthreads();
-      cg_dev<D>(m, T, eps, W, Mout, Y, reinterpret_cast<double*>(cgws) + (long long)bh * 4 * md, reinterpret_cast<double*>(dyn_smem), red);
-      if (dev_status) {
-        float bad = 0.f;
-        for (int e = tid; e < m * D; e += 256) bad += isfinite(Y[e]) ? 0.f : 1.f;
-        bad = block_sum(bad, red);
-        if (tid == 0 && bad > 0.f) atomicOr(dev_status + bh, 1);
-      }
+  if constexpr (CG) {
+    static_assert(!TC && MP == 0 && CL == 1, "one CTA per head");
+    __syncthreads();
+    cg_dev<D>(m, T, eps, W, Mout, Y, reinterpret_cast<double*>(cgws) + (long long)bh * 4 * md, reinterpret_cast<double*>(dyn_smem), red);
+    if (dev_status) {
+      float bad = 0.f;
+      for (int e = tid; e < m * D; e += 256) bad += isfinite(Y[e]) ? 0.f : 1.f;
+      bad = block_sum(bad, red);
+      if (tid == 0 && bad > 0.f) atomicOr(dev_status + bh, 1);
     }
   } else if constexpr (MP == 256) {               // Y = X M on the engine of the iteration (images of X_T in Wr, of M in P)
     if (!(phase & 1)) u2_begin(u2c, ctl256, mbars256, reinterpret_cast<bf16*>(dyn_smem), 256);
@@ -2244,19 +2286,19 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
     gu_write_images(Yt, Yimg + (long long)bh * nkb * (2 * GU_KB * D), m, D, gt, gn);
   }
 }
-template <int D, bool TC, int MP, int CL = 1>
+template <int D, bool TC, int MP, int CL = 1, bool CG = false>
 __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 : 1)) k_mid_bwd(int m, int T, int H, int map_mode, float inv_lambda, int ldm,
                                                  const float* __restrict__ whiten, const float* W,
                                                  const float* Xh, const float* Ph, const NsHdr* hdr, const float* Msaved,
                                                  const float* dYtpart, const float* dybpart, int nchunks,
                                                  float eps, float* Wr, float* P, float* Hm, float* Ga, float* Gb,
                                                  float* dWm, float* dXm, float* dY, float* dM, float* GW, int* dev_status,
-                                                 long long hslot, bf16* dMimg, int sym, int solver = 0, const float* Ysaved = nullptr,
+                                                 long long hslot, bf16* dMimg, int sym, const float* Ysaved = nullptr,
                                                  float* cgws = nullptr, int phase = 3) {
   pdl_wait();
   // phase: bit 0 = dY, dX and dM (what the key-side kernels wait for), bit 1 = the adjoint of the iteration and GW.
   // The two halves may run as two launches on one stream: the key-side sign pass then starts after the first.
-  // solver 1 (conjugate gradients, the fp32 single-CTA instantiation only): the solve is differentiated as the linear
+  // CG (conjugate gradients, see k_mid_fwd): the solve is differentiated as the linear
   // system it approximates, dM = the T-step iterate of (W + eps I) dM = dY, dW = -dM Y^T (Ysaved: Y of the forward pass)
   // sym: 1 = one landmark set (W = k(L, L): the gradient of both roles of L is carried by the symmetrised factor);
   // 0 = two landmark sets, GW = dW o W / lambda as it is (MP == 0 only)
@@ -2322,11 +2364,10 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
   }
   phase_sync<CL>();
   const float* XT = Xh + (long long)T * mx;
-  if (solver == 1) {
-    if constexpr (!TC && MP == 0 && CL == 1) {
-      cg_dev<D>(m, T, eps, W, dY, dM, reinterpret_cast<double*>(cgws) + (long long)bh * 4 * md, reinterpret_cast<double*>(dyn_smem), red);
-      ns_gemm<TC, false, true>(m, m, D, dM, D, Ysaved + bh * md, D, dWm, ldx, -1.f, 0.f, nullptr, 0.f, sm, crank, CL);   // dW = -dM Y^T
-    }
+  if constexpr (CG) {
+    static_assert(!TC && MP == 0 && CL == 1, "one CTA per head");
+    cg_dev<D>(m, T, eps, W, dY, dM, reinterpret_cast<double*>(cgws) + (long long)bh * 4 * md, reinterpret_cast<double*>(dyn_smem), red);
+    cg_dw<D>(m, dM, Ysaved + bh * md, dWm, ldx, reinterpret_cast<float*>(dyn_smem));   // dW = -dM Y^T
   } else if constexpr (MP == 256) {                  // dX = dY M^T and dM = X^T dY on the engine of the adjoint
     u2_begin(u2c, ctl256, mbars256, reinterpret_cast<bf16*>(dyn_smem), 512);
     const bool p_ok = u2_products_dx_dm(u2c, m, D, dY, Msaved, XT, Hm, Gb, dXm, dM, crank);
@@ -2354,7 +2395,7 @@ __global__ void __launch_bounds__(256, MP == 64 ? 3 : ((CL > 1 && MP == 0) ? 2 :
     umma::report_timeout(tc_ok, dev_status, bh);
     // end of the adjoint and GW in one pass (the operand buffers are free: the engine has ended with a cluster barrier)
     ns_tail_gw_sym<CL>(m, ldm, W, eps, hdr, P, dWm, inv_lambda, GW, red, reinterpret_cast<float*>(dyn_smem), crank);
-  } else if (solver == 0) { ns_backward_dev<TC, CL>(m, T, Wr, Xh, hdr, dXm, dWm, P, Hm, Ga, Gb, sm, red, crank, Ph); if (CL > 1) phase_sync<CL>(); }
+  } else if constexpr (!CG) { ns_backward_dev<TC, CL>(m, T, Wr, Xh, hdr, dXm, dWm, P, Hm, Ga, Gb, sm, red, crank, Ph); if (CL > 1) phase_sync<CL>(); }
   // GW = (dW o K_LL + (dW o K_LL)^T) / lambda; four elements per batch so that the loads overlap
   // (the tcgen05 engines have written GW already)
   if constexpr (MP == 0)
