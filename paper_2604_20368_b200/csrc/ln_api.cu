@@ -456,7 +456,21 @@ CopyStreams copy_acquire(cudaStream_t caller) {
 }
 
 // Launch with `cl` CTAs per thread-block cluster (cl = 1: an ordinary launch).
-constexpr int kMidCluster = 4;     // CTAs that share one head on the general (two landmark sets) engine beyond 64 landmarks
+// CTAs that share one head beyond 64 landmarks on the engines that keep their matrices in global memory: the mma.sync engine
+// (two landmark sets, bf16 storage) and the FFMA engine (fp32 storage).  Four give the shorter chain.  The FFMA engine takes
+// two where that gives fewer (waves of the grid at two CTAs per SM) x (rounds of 64 x 64 output tiles per product); of the
+// places, clusters of four get thirteen fourteenths (68 heads are resident, 72 not), clusters of two all.  On a tie the
+// fixed part of a product decides, which counts up to about 128 landmarks.  fp32 inference, 400 tokens per head, 64 dims,
+// four / two CTAs per head (one, before the engine was shared): 65 landmarks, 68 heads 237 / 258 us (339), 148 heads
+// 521 / 419 (432), 152 heads 539 / 560 (657), 256 heads 829 / 770 (788); 150 landmarks, 96 heads 1083 / 1133 (1245), 148 heads
+// 1613 / 1223 (1358); 256 landmarks, 96 heads 1904 / 2280 (3409), 148 heads 2969 / 2420 (3874).
+constexpr int kMidCluster = 4;
+inline int mid_cluster_f32(int heads, int m) {
+  const long long sms = sm_count(), t = (m + 63) / 64;
+  auto cost = [&](long long cl, long long resident) { return (heads + resident - 1) / resident * ((t * t + cl - 1) / cl); };
+  const long long c4 = cost(4, 2 * sms * 13 / 14 / 4), c2 = cost(2, sms);
+  return c4 < c2 || (c4 == c2 && m >= 128) ? kMidCluster : 2;
+}
 template <typename... KArgs, typename... Args>
 void launch_clustered(void (*kern)(KArgs...), int grid, int cl, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -577,7 +591,8 @@ int fwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
     const size_t mid_smem = TC ? sizeof(MmaGemmSmem) : (m <= 64 && kResFwdSmem > sizeof(GemmSmem) ? kResFwdSmem : sizeof(GemmSmem));
     // two landmark sets (general matrix) or fp32 storage: the mma.sync or FFMA engine, shared by the CTAs of a cluster
     // beyond 64 landmarks
-    if ((two || !TC) && m > 64) launch(k_mid_fwd<D, TC, 0, kMidCluster>, mid_smem, kMidCluster);
+    if (!TC && m > 64 && mid_cluster_f32(BH, m) == 2) launch(k_mid_fwd<D, TC, 0, TC ? kMidCluster : 2>, mid_smem, 2);
+    else if ((two || !TC) && m > 64) launch(k_mid_fwd<D, TC, 0, kMidCluster>, mid_smem, kMidCluster);
     else if (two) launch(k_mid_fwd<D, TC, 0>, mid_smem);
     else if (TC && m <= 64) launch(k_mid_fwd<D, TC, TC ? 64 : 0>, 3 * kUmmaMatBytes64);
     else if (TC && m <= 128) launch(k_mid_fwd<D, TC, TC ? 128 : 0>, 3 * kUmmaMatBytes);
@@ -744,7 +759,8 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
     };
     const size_t mid_smem = TC ? sizeof(MmaGemmSmem) : (m <= 64 ? kResBwdSmem : sizeof(GemmSmem));
     if (pl.cg) { launch(k_mid_bwd<D, false, 0, 1, true>, kCgSmem); return; }
-    if ((two || !TC) && m > 64) launch(k_mid_bwd<D, TC, 0, kMidCluster>, mid_smem, kMidCluster);
+    if (!TC && m > 64 && mid_cluster_f32(BH, m) == 2) launch(k_mid_bwd<D, TC, 0, TC ? kMidCluster : 2>, mid_smem, 2);
+    else if ((two || !TC) && m > 64) launch(k_mid_bwd<D, TC, 0, kMidCluster>, mid_smem, kMidCluster);
     else if (two) launch(k_mid_bwd<D, TC, 0>, mid_smem);
     else if (TC && m <= 64) launch(k_mid_bwd<D, TC, TC ? 64 : 0>, 4 * kUmmaMatBytes64);
     else if (TC && m <= 128) launch(k_mid_bwd<D, TC, TC ? 128 : 0>, 3 * kUmmaMatBytes);

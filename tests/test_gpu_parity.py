@@ -360,6 +360,14 @@ def test_fp32_storage_path_over_the_solver_variants(mh, mw):
     _run_case(cfg)
 
 
+@pytest.mark.parametrize("mh,mw,B", [(5, 13, 17), (5, 13, 36), (8, 16, 36), (10, 13, 36), (15, 17, 18)])
+def test_fp32_storage_path_with_many_heads(mh, mw, B):
+    """68 to 144 heads beyond 64 landmarks: clusters of four per head while all are resident, of two where that saves a wave
+    of the grid."""
+    cfg = synth.Config("f32_many", B=B, H=4, d=32, m=mh * mw, T=4, gh=20, gw=20, mh=mh, mw=mw, prefix=1, dtype="f32", seed=11 + B)
+    _run_case(cfg, heads=[0, 4 * B - 1])
+
+
 # Ragged shapes for the fused sign pass (token tiles of 8 * TG tokens, rounds of 8 landmarks, several token
 # chunks per head, two 64-dim slabs) and for the per-head kernels (m <= 64, 64 < m <= 128, clustered m > 128).
 @pytest.mark.parametrize("gh,gw,mh,mw,prefix,d,dtype", [
