@@ -110,8 +110,7 @@ typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 add2(f32x2 x, f32x2 y) { f32x2 z; asm("add.f32x2 %0, %1, %2;" : "=l"(z) : "l"(x), "l"(y)); return z; }
 __device__ __forceinline__ f32x2 fma2(f32x2 x, f32x2 y, f32x2 c) { f32x2 z; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(z) : "l"(x), "l"(y), "l"(c)); return z; }
 __device__ __forceinline__ f32x2 mul2(f32x2 x, f32x2 y) { f32x2 z; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(z) : "l"(x), "l"(y)); return z; }
-// Halves of a pair and a pair from two halves, written as register-pair moves: spelled with 64-bit shifts and ORs the
-// compiler emits real integer instructions for them, which cost issue slots in the FP32-bound inner loops.
+// Halves of a pair and a pair from two halves: a pair is a pair of registers, so these are moves, not shifts.
 __device__ __forceinline__ float lo32(f32x2 x) { float a, b; asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x)); return a; }
 __device__ __forceinline__ float hi32(f32x2 x) { float a, b; asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x)); return b; }
 __device__ __forceinline__ f32x2 pack2(float a, float b) { f32x2 z; asm("mov.b64 %0, {%1, %2};" : "=l"(z) : "f"(a), "f"(b)); return z; }

@@ -1326,7 +1326,7 @@ union __align__(16) NsSmem { GemmSmem f; MmaGemmSmem t; };
 
 // C = beta*Cin + alpha*op(A)op(B) + diag*I on either engine: TC = tensor cores with split-bf16
 // operands (bf16-storage path), else exact fp32 FFMA (fp32-storage path, stand-alone ns_pinv).
-template <bool TC, bool TRA, bool TRB, bool BIG = false>
+template <bool TC, bool TRA, bool TRB>
 __device__ __forceinline__ void ns_gemm(int M, int N, int K, const float* A, int lda, const float* Bm, int ldb,
                                         float* C, int ldc, float alpha, float beta, const float* Cin, float diag,
                                         NsSmem& sm, int part = 0, int nparts = 1) {
@@ -1341,7 +1341,7 @@ __device__ __forceinline__ void ns_gemm(int M, int N, int K, const float* A, int
 // fp32 Newton-Schulz and its adjoint for m <= 64 by one CTA, every matrix of a step resident in shared memory (row-major,
 // pitch 68: all four transpose variants of a product read it without bank conflicts).  A product is then no longer a
 // round trip through L2: thread (ty, tx) of one of four groups of 64 threads forms rows ty + 8 r, columns tx + 8 q
-// (r, q < NR = 4, 7 or 8, whichever hugs m) over its quarter of k, and the four partial sums are added in a fixed order.
+// (r, q < NR = 4, 7 or 8 for m <= 32, 56, 64) over its quarter of k, and the four partial sums are added in a fixed order.
 // At m = 49, T = 6, 32 heads: k_mid_fwd / k_mid_bwd 72 / 141 -> 50 / 93 us (2.2 us a product instead of 4.0).
 // =====================================================================================
 constexpr int RS_P = 68;                          // pitch of a resident matrix
@@ -1684,9 +1684,9 @@ __device__ void ns_forward_dev(int m, int T, float eps, float alpha_in, const fl
     const float* X = Xh + (long long)k * mm;
     float* Xn = Xh + (long long)(k + 1) * mm;
     float* Q = Qh ? Qh + (long long)k * mm : P;
-    ns_gemm<TC, false, false, true>(m, m, m, Wr, m, X, m, Q, m, -1.f, 0.f, nullptr, 2.f, sm, crank, CL);   // Q = 2I - Wr X_k
+    ns_gemm<TC, false, false>(m, m, m, Wr, m, X, m, Q, m, -1.f, 0.f, nullptr, 2.f, sm, crank, CL);   // Q = 2I - Wr X_k
     if (CL > 1) phase_sync<CL>();
-    ns_gemm<TC, false, false, true>(m, m, m, X, m, Q, m, Xn, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);    // X_{k+1} = X_k Q
+    ns_gemm<TC, false, false>(m, m, m, X, m, Q, m, Xn, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);    // X_{k+1} = X_k Q
     if (CL > 1) phase_sync<CL>();
   }
 }
@@ -1723,14 +1723,14 @@ __device__ void ns_backward_dev(int m, int T, const float* Wr, const float* Xh, 
     const float* A = Xh + (long long)k * mm;                                        // X_{k+1} = 2A - A P, P = Wr A
     const float* dWin = k == T - 1 ? nullptr : dW;                                  // the first step starts the sum
     const float b1 = dWin ? 1.f : 0.f;
-    if (!Qh) ns_gemm<TC, false, false, true>(m, m, m, Wr, m, A, m, P, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);      // P = Wr A
-    ns_gemm<TC, true, false, true>(m, m, m, A, m, G, m, Hm, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);       // H = A^T G
+    if (!Qh) ns_gemm<TC, false, false>(m, m, m, Wr, m, A, m, P, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);      // P = Wr A
+    ns_gemm<TC, true, false>(m, m, m, A, m, G, m, Hm, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);       // H = A^T G
     if (CL > 1) phase_sync<CL>();
-    ns_gemm<TC, false, true, true>(m, m, m, Hm, m, A, m, dW, m, -1.f, b1, dWin, 0.f, sm, crank, CL);         // dW -= H A^T
+    ns_gemm<TC, false, true>(m, m, m, Hm, m, A, m, dW, m, -1.f, b1, dWin, 0.f, sm, crank, CL);         // dW -= H A^T
     if constexpr (TC) {
-      if (Qh) ns_gemm<TC, false, true, true>(m, m, m, G, m, Qh + (long long)k * mm, m, Gn, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);   // Gn = G Q^T
-      else ns_gemm<TC, false, true, true>(m, m, m, G, m, P, m, Gn, m, -1.f, 2.f, G, 0.f, sm, crank, CL);     // Gn = 2G - G P^T
-      ns_gemm<TC, true, false, true>(m, m, m, Wr, m, Hm, m, Gn, m, -1.f, 1.f, Gn, 0.f, sm, crank, CL);       // Gn -= Wr^T H
+      if (Qh) ns_gemm<TC, false, true>(m, m, m, G, m, Qh + (long long)k * mm, m, Gn, m, 1.f, 0.f, nullptr, 0.f, sm, crank, CL);   // Gn = G Q^T
+      else ns_gemm<TC, false, true>(m, m, m, G, m, P, m, Gn, m, -1.f, 2.f, G, 0.f, sm, crank, CL);     // Gn = 2G - G P^T
+      ns_gemm<TC, true, false>(m, m, m, Wr, m, Hm, m, Gn, m, -1.f, 1.f, Gn, 0.f, sm, crank, CL);       // Gn -= Wr^T H
     } else {                                                                        // both terms in one accumulation
       const FgSecond wh = {Wr, m, Hm, m, m};
       if (Qh) cta_gemm<false, true, true, true, false, true>(m, m, m, G, m, Qh + (long long)k * mm, m, Gn, m, 1.f, 0.f, nullptr, 0.f, sm.f, crank, CL, wh);

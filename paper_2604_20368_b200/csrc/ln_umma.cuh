@@ -45,11 +45,10 @@ __device__ __forceinline__ uint32_t instr_desc(int N, bool a_mn_major, bool b_mn
 }
 
 // The one thread of a CTA (of the warp) that issues tensor-core and bulk-copy instructions; the same thread at every call.
-// tcgen05.mma takes its operands from uniform registers.  Behind elect.sync the compiler knows that one lane is active
-// and moves them there directly; behind a test of threadIdx it has to cover the case of several lanes with different
-// operands and wraps every instruction in a loop: 165 to 208 clocks per MMA, whatever its size, against the 9 (N = 16)
-// to 64 (N = 128) the tensor core takes (measured with 4096 MMAs in a row per SM, run-time shapes).  In the kernels,
-// whose loops are unrolled, the step took k_mid_fwd / k_mid_bwd at m = 256 from 923 / 1673 to 886 / 1580 us.
+// elect.sync is the way to single out one lane of a converged warp for these instructions.  Behind it an MMA issues in
+// the 9 (N = 16) to 64 (N = 128) clocks that the tensor core takes; behind a test of threadIdx it took 165 to 208, whatever
+// its size (4096 MMAs in a row per SM, run-time shapes).  In the kernels k_mid_fwd / k_mid_bwd at m = 256 went from 923 / 1673
+// to 886 / 1580 us.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
