@@ -124,6 +124,16 @@ bool make_plan(const ln_problem* p, Plan* pl) {
   if (want < 1) want = 1;
   int rpc = (p->n + want - 1) / want;
   if (rpc < 256) rpc = 256;
+  // fp32 storage: where chunks of 256 tokens are fewer than two CTAs per SM the product is a chain of eight 32-token steps on
+  // a part of the chip; shorter chunks then, down to 64 tokens and for up to three CTAs per SM (three heads x 196 tokens
+  // 3 -> 12 CTAs, 32 heads x 784 tokens 128 -> 416; figures at k_tn).  bf16 storage keeps its chunks: its ring of three
+  // stages hides the loads, and the order of its sums stays as it was.
+  if (p->dtype == LN_F32 && (long long)pl->BH * mblk * ((p->n + rpc - 1) / rpc) < 2ll * kSMs) {
+    int parts = (3 * kSMs + pl->BH * mblk - 1) / (pl->BH * mblk);
+    if (parts > 32) parts = 32;
+    const int shorter = (p->n + parts - 1) / parts;
+    rpc = shorter < 64 ? 64 : (shorter < rpc ? shorter : rpc);
+  }
   rpc = (rpc + 31) / 32 * 32;
   pl->rpc = rpc;
   pl->chunks = (p->n + rpc - 1) / rpc;

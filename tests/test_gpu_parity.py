@@ -360,6 +360,15 @@ def test_fp32_storage_path_over_the_solver_variants(mh, mw):
     _run_case(cfg)
 
 
+@pytest.mark.parametrize("gh,gw,prefix,d", [(7, 9, 0, 64), (8, 8, 0, 32), (5, 13, 0, 64), (16, 8, 1, 128), (15, 17, 1, 64), (20, 33, 0, 32)])
+@pytest.mark.parametrize("B", [1, 40])
+def test_fp32_storage_token_chunks(gh, gw, prefix, d, B):
+    """Sums over the tokens (M = R V, Z'^T dO) in chunks of 64 tokens where few heads leave the GPU empty, longer ones for many
+    heads: one chunk, a remainder of one token, whole and odd numbers of chunks."""
+    cfg = synth.Config("f32_chunks", B=B, H=3, d=d, m=20, T=4, gh=gh, gw=gw, mh=4, mw=5, prefix=prefix, dtype="f32", seed=77 + gh)
+    _run_case(cfg, heads=[0, 3 * B - 1], intermediates=True)
+
+
 @pytest.mark.parametrize("mh,mw,B", [(5, 13, 17), (5, 13, 36), (8, 16, 36), (10, 13, 36), (15, 17, 18)])
 def test_fp32_storage_path_with_many_heads(mh, mw, B):
     """68 to 144 heads beyond 64 landmarks: clusters of four per head while all are resident, of two where that saves a wave
