@@ -958,6 +958,33 @@ __global__ void __launch_bounds__(256) k_nt_g(const TU* __restrict__ U, const fl
   }
 }
 
+// Eight consecutive entries of a row of an [.][ld] matrix, zero from `end` on.  vec: rows and base are 16-byte aligned.
+__device__ __forceinline__ void sign_fetch8(const float* __restrict__ row, bool vec, bool in, int l, int end, float (&v)[8]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int q = l + 4 * h;
+    if (in && vec && q + 3 < end) {
+      const float4 g = ld4(row + q);
+      v[4 * h] = g.x; v[4 * h + 1] = g.y; v[4 * h + 2] = g.z; v[4 * h + 3] = g.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[4 * h + e] = (in && q + e < end) ? row[q + e] : 0.f;
+    }
+  }
+}
+// The upstream factor: G, times the kernel value over lambda where that is given.  Formed where the tile is stored, so that
+// nothing waits for the loads before the step in front of it has run.
+__device__ __forceinline__ void sign_store8(float* dst, const float (&g)[8], const float (&w)[8], bool mul, float gscale) {
+  float v[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) v[e] = mul ? g[e] * (w[e] * gscale) : g[e];
+  *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+  *reinterpret_cast<float4*>(dst + 4) = make_float4(v[4], v[5], v[6], v[7]);
+}
+__device__ __forceinline__ bool sign_vec(const float* G, const float* Gk, int ldg) {
+  return (ldg & 3) == 0 && ((reinterpret_cast<uintptr_t>(G) | reinterpret_cast<uintptr_t>(Gk)) & 15) == 0;
+}
+
 // =====================================================================================
 // Sign pass over the landmarks (App. A):  out[i][c] = -sum_l G[i][l] * sign(tok[i][c] - L[l][c])
 // grid (ceil(n/64), BH[, splits]); thread: 4 tokens x D/16 dims, token values held in registers.
@@ -996,24 +1023,34 @@ __global__ void __launch_bounds__(256) k_sign_rows(const TT* __restrict__ tok, c
       qp[k][s] = pack2(q0, q1);
     }
   }
+  // The tile of the next step (32 landmarks; 64 tokens x 32 entries of G) is on its way to registers during this one, G in
+  // quads where rows are aligned: eight 4-byte loads per thread and matrix, 32 bytes apart between lanes, touched every
+  // sector eight times.  l1_kernel + l1_kernel_bwd on two 1024 x 1024 blocks with 32 dims 49.1 -> 42.1 us, same bits.
+  const bool vec = sign_vec(G, Gk, ldg);
+  float4 lv[D / 32];
+  float gv[8], kv[8];
+  auto fetch = [&](int l0) {
+#pragma unroll
+    for (int t = 0; t < D / 32; ++t) {
+      const int idx = tid + t * 256, r = idx / (D / 4), c4 = (idx % (D / 4)) * 4;
+      lv[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (l0 + r < lend) lv[t] = ld4(Lm + (long long)(l0 + r) * D + c4);
+    }
+    const int i = i0 + (tid >> 2);
+    const long long row = (long long)(i < n ? i : 0) * ldg;
+    sign_fetch8(G + row, vec, i < n, l0 + (tid & 3) * 8, lend, gv);
+    if (Gk) sign_fetch8(Gk + row, vec, i < n, l0 + (tid & 3) * 8, lend, kv);
+  };
+  if (lbeg < lend) fetch(lbeg);
   for (int l0 = lbeg; l0 < lend; l0 += 32) {
     __syncthreads();
-    for (int idx = tid; idx < 32 * (D / 4); idx += 256) {
-      const int r = idx / (D / 4), c4 = (idx % (D / 4)) * 4;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (l0 + r < lend) v = ld4(Lm + (long long)(l0 + r) * D + c4);
-      *reinterpret_cast<float4*>(&Ls[r][c4]) = make_float4(-v.x, -v.y, -v.z, -v.w);   // negated: q - L is a packed add
-    }
-    {  // G tile: 64 tokens x 32 landmarks (zero outside)
-      const int r = tid >> 2, cb = (tid & 3) * 8, i = i0 + r;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int l = l0 + cb + k;
-        float gv = (i < n && l < lend) ? G[(long long)i * ldg + l] : 0.f;
-        if (Gk && i < n && l < lend) gv *= Gk[(long long)i * ldg + l] * gscale;
-        Gs[r][cb + k] = gv;
-      }
+    for (int t = 0; t < D / 32; ++t) {       // negated: q - L is a packed add
+      const int idx = tid + t * 256;
+      *reinterpret_cast<float4*>(&Ls[idx / (D / 4)][(idx % (D / 4)) * 4]) = make_float4(-lv[t].x, -lv[t].y, -lv[t].z, -lv[t].w);
     }
+    sign_store8(&Gs[tid >> 2][(tid & 3) * 8], gv, kv, Gk != nullptr, gscale);
+    if (l0 + 32 < lend) fetch(l0 + 32);
     __syncthreads();
     const int lcount = min(32, (lend - l0 + 3) & ~3);  // landmarks of this chunk, rounded up to 4 (the rest is zero)
 #pragma unroll 2
@@ -1085,24 +1122,32 @@ __global__ void __launch_bounds__(256) k_sign_cols(const TT* __restrict__ tok, c
       nl[k][s] = pack2(-v0, -v1);
     }
   }
+  // as in the pass over the landmarks: the next tile (32 tokens; 32 x 64 entries of G) on its way during this one
+  const bool vec = sign_vec(G, Gk, ldg);
+  float4 tk[D / 32];
+  float gv[8], kv[8];
+  auto fetch = [&](int j0) {
+#pragma unroll
+    for (int t = 0; t < D / 32; ++t) {
+      const int idx = tid + t * 256, r = idx / (D / 4), c4 = (idx % (D / 4)) * 4;
+      tk[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (j0 + r < iend) tk[t] = ld4(tok + (long long)(j0 + r) * D + c4);
+    }
+    const int i = j0 + (tid >> 3);
+    const long long row = (long long)(i < iend ? i : 0) * ldg;
+    sign_fetch8(G + row, vec, i < iend, l0 + (tid & 7) * 8, m, gv);
+    if (Gk) sign_fetch8(Gk + row, vec, i < iend, l0 + (tid & 7) * 8, m, kv);
+  };
+  if (ibeg < iend) fetch(ibeg);
   for (int j0 = ibeg; j0 < iend; j0 += 32) {
     __syncthreads();
-    for (int idx = tid; idx < 32 * (D / 4); idx += 256) {
-      const int r = idx / (D / 4), c4 = (idx % (D / 4)) * 4;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (j0 + r < iend) v = ld4(tok + (long long)(j0 + r) * D + c4);
-      *reinterpret_cast<float4*>(&Ts[r][c4]) = v;
-    }
-    {  // G tile: 32 tokens x 64 landmarks (zero outside)
-      const int r = tid >> 3, cb = (tid & 7) * 8, i = j0 + r;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int l = l0 + cb + k;
-        float gv = (i < iend && l < m) ? G[(long long)i * ldg + l] : 0.f;
-        if (Gk && i < iend && l < m) gv *= Gk[(long long)i * ldg + l] * gscale;
-        Gs[r][cb + k] = gv;
-      }
+    for (int t = 0; t < D / 32; ++t) {
+      const int idx = tid + t * 256;
+      *reinterpret_cast<float4*>(&Ts[idx / (D / 4)][(idx % (D / 4)) * 4]) = tk[t];
     }
+    sign_store8(&Gs[tid >> 3][(tid & 7) * 8], gv, kv, Gk != nullptr, gscale);
+    if (j0 + 32 < iend) fetch(j0 + 32);
     __syncthreads();
     const int jcount = min(32, iend - j0);
 #pragma unroll 4
