@@ -1025,14 +1025,15 @@ void l1_bwd_impl(int batch, int na, int nb, const T* A, const T* Bm, float lambd
   if (!Kmat) { launch_l1<T, T>("l1_kernel", A, Bm, w.Kmat, nullptr, batch, na, nb, D, nb, lambda, st); Kmat = w.Kmat; }
   // the factor dK o K / lambda is formed where the two passes load their tiles of it
   const float il = 1.f / lambda;
+  const int rowtiles = (int)cdiv(na, 64);
+  const dim3 grid(rowtiles * w.lsplits + w.chunks * cdiv(nb, 64), batch);
   if (w.lsplits > 1) {
-    LN_LAUNCH("k_sign_rows", st, enqueue(k_sign_rows<T, T, float, D>, dim3(cdiv(na, 64), batch, w.lsplits), 256, 0, st, A, Bm, dK, nb, w.rowpart, na, nb, w.lper, Kmat, il));
-    LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3<T>, dim3(cdiv(na * D, 1024), batch), 256, 0, st, w.rowpart, w.lsplits, nullptr, 0, nullptr, 0, dA, na * D));
+    LN_LAUNCH("k_sign_both", st, enqueue(k_sign_both<T, float, D>, grid, 256, 0, st, A, Bm, dK, Kmat, il, w.rowpart, w.part, na, nb, rowtiles, w.lsplits, w.lper, w.chunks, w.rpc));
+    LN_LAUNCH("k_reduce_two", st, enqueue(k_reduce_two<T>, dim3(cdiv((na > nb ? na : nb) * D, 1024), batch, 2), 256, 0, st, w.rowpart, w.lsplits, dA, na * D, w.part, w.chunks, dB, nb * D));
   } else {
-    LN_LAUNCH("k_sign_rows", st, enqueue(k_sign_rows<T, T, T, D>, dim3(cdiv(na, 64), batch), 256, 0, st, A, Bm, dK, nb, dA, na, nb, 0, Kmat, il));
+    LN_LAUNCH("k_sign_both", st, enqueue(k_sign_both<T, T, D>, grid, 256, 0, st, A, Bm, dK, Kmat, il, dA, w.part, na, nb, rowtiles, 1, 0, w.chunks, w.rpc));
+    LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3<T>, dim3(cdiv(nb * D, 1024), batch), 256, 0, st, w.part, w.chunks, nullptr, 0, nullptr, 0, dB, nb * D));
   }
-  LN_LAUNCH("k_sign_cols", st, enqueue(k_sign_cols<T, T, D>, dim3(w.chunks, cdiv(nb, 64), batch), 256, 0, st, A, Bm, dK, nb, w.part, na, nb, w.rpc, Kmat, il));
-  LN_LAUNCH("k_reduce3", st, enqueue(k_reduce3<T>, dim3(cdiv(nb * D, 1024), batch), 256, 0, st, w.part, w.chunks, nullptr, 0, nullptr, 0, dB, nb * D));
 }
 }  // namespace
 
