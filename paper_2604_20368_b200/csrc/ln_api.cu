@@ -67,15 +67,27 @@ struct Carver {
 // Tile of the l1 kernel for a problem: LG landmark groups of QN (4 or 2) landmarks, TG token groups of 8,
 // LG * TG <= 256 threads, chosen so that the tiles hug the problem.  Small heads (few pairs per CTA) take
 // the two-landmark thread tile, which fits three CTAs per SM.
+// CTAs of up to 128 threads (four or six per SM; `fine`): more of them are at different points of load, barrier and arithmetic,
+// and the tiles are finer.  They are taken where they fill their warps and cover the tokens about as well as CTAs of 256 (m = 49
+// with four landmarks a thread does not: 13 x 9 threads of 128 against 13 x 19 of 256), and only for launches that have the GPU
+// to themselves or outlast what runs beside them (see launch_l1_args).
 struct L1Launch { dim3 grid, block; size_t smem; int qn; };
-L1Launch plan_l1(int na_max, int nb, int d, int batch, int nprob) {
+L1Launch plan_l1(int na_max, int nb, int d, int batch, int nprob, bool fine) {
   const int qn = ((long long)na_max * nb * d <= (1ll << 20)) ? 2 : 4;
   const int lg_cap = (qn == 4) ? 16 : 32;
   int LG = (nb + qn - 1) / qn; if (LG > lg_cap) LG = lg_cap; if (LG < 1) LG = 1;
-  int tg_cap = 256 / LG; if (tg_cap > 32) tg_cap = 32;       // at most 256 tokens per tile
   const int groups = (na_max + 7) / 8;
-  const int tiles = (groups + tg_cap - 1) / tg_cap;
-  int TG = (groups + tiles - 1) / tiles; if (TG < 1) TG = 1;
+  // token groups of a CTA of up to `cap` threads (at most 256 tokens) and the share of its lanes' time that is of use
+  auto fit = [&](int cap, int& TG) {
+    int tg_cap = cap / LG; if (tg_cap > 32) tg_cap = 32;
+    const int tiles = (groups + tg_cap - 1) / tg_cap;
+    TG = (groups + tiles - 1) / tiles; if (TG < 1) TG = 1;
+    const int threads = LG * TG, ctas = (na_max + 8 * TG - 1) / (8 * TG);
+    return (double)threads / ((threads + 31) / 32 * 32) * na_max / ((double)ctas * 8 * TG);
+  };
+  int TG, TGs;
+  const double large = fit(256, TG), small = fit(128, TGs);
+  if (fine && small >= 0.98 * large) TG = TGs;
   L1Launch l;
   l.qn = qn;
   l.block = dim3(LG, TG);
@@ -176,7 +188,7 @@ bool make_plan(const ln_problem* p, Plan* pl) {
   }
   // bf16 storage, 64 or 128 dims: one CTA per tile of 8 * TG tokens, upstream factor on the tensor cores in the kernel
   pl->H = p->H; pl->wmode = p->whiten_mode;
-  pl->l1_tiles = (int)plan_l1(p->n, p->m, p->d, pl->BH, 1).grid.x;
+  pl->l1_tiles = (int)plan_l1(p->n, p->m, p->d, pl->BH, 1, false).grid.x;
   pl->s3_tiles = (p->dtype == LN_BF16 && (p->d == 64 || p->d == 128) && g_sign3.load(std::memory_order_relaxed))
                      ? (p->n + 8 * pl->s2_tg - 1) / (8 * pl->s2_tg) : 0;
   return true;
@@ -521,7 +533,14 @@ L1Prob l1_prob(const void* A, int a_f32, float* E, float* rowsum, int na, int d,
 void launch_l1_args(const char* name, L1Args& a, int nprob, int batch, cudaStream_t st) {
   int na_max = 0;
   for (int i = 0; i < nprob; ++i) na_max = a.p[i].na > na_max ? a.p[i].na : na_max;
-  L1Launch l = plan_l1(na_max, a.nb, a.d, batch, nprob);
+  // Smaller CTAs where C, R^T and W are one launch (nothing runs beside it), or from 2^30 (pair, dim)s on: 384 heads x 197
+  // tokens, 49 landmarks 82.7 -> 76.6 us (step 466 -> 461); 224 x 224-token inference 1546 -> 1520 us, step of 128 heads with 256
+  // landmarks 12758 -> 12699.  Shorter launches beside the per-head kernels lose: their CTAs take the places these wait for
+  // (step of 32 x 3136 tokens 397 -> 399, of 15 x 1074 tokens 187 -> 190).  The partial column statistics have one slot per
+  // tile of the larger CTAs.
+  bool fine = nprob == 3 || (long long)na_max * a.nb * a.d * batch > (1ll << 30);
+  for (int i = 0; i < nprob; ++i) fine = fine && !a.p[i].stat;
+  L1Launch l = plan_l1(na_max, a.nb, a.d, batch, nprob, fine);
   // a single block without row sums (the stand-alone entry point on few, large matrices): the landmark range is split
   // over blockIdx.z until the launch has about two CTAs per SM
   a.jsplits = 1;

@@ -369,6 +369,16 @@ def test_fp32_storage_token_chunks(gh, gw, prefix, d, B):
     _run_case(cfg, heads=[0, 3 * B - 1], intermediates=True)
 
 
+@pytest.mark.parametrize("mh,mw", [(1, 1), (2, 3), (3, 5), (5, 5), (7, 7), (8, 8)])
+@pytest.mark.parametrize("gh,gw,prefix,d,dtype,B", [(8, 8, 1, 64, "f32", 1), (9, 14, 0, 32, "f32", 2), (14, 14, 1, 64, "bf16", 56),
+                                                    (9, 8, 0, 128, "bf16", 56)])
+def test_kernel_blocks_in_one_launch(mh, mw, gh, gw, prefix, d, dtype, B):
+    """C, R^T and W from one launch (fp32 storage, or more than 220 bf16 heads of few tokens), whose CTAs have up to 128 threads
+    where these fill their warps: one to 49 landmark groups, token tiles with and without a remainder."""
+    cfg = synth.Config("one_launch", B=B, H=4, d=d, m=mh * mw, T=3, gh=gh, gw=gw, mh=mh, mw=mw, prefix=prefix, dtype=dtype, seed=5 + mh * mw)
+    _run_case(cfg, heads=[0, 4 * B - 1], intermediates=True)
+
+
 @pytest.mark.parametrize("mh,mw,B", [(5, 13, 17), (5, 13, 36), (8, 16, 36), (10, 13, 36), (15, 17, 18)])
 def test_fp32_storage_path_with_many_heads(mh, mw, B):
     """68 to 144 heads beyond 64 landmarks: clusters of four per head while all are resident, of two where that saves a wave
