@@ -843,37 +843,50 @@ __global__ void __launch_bounds__(256) k_nn(const float* __restrict__ E, int lde
 #pragma unroll
     for (int q = 0; q < DC; ++q) acc[k][q] = 0.f;
 
+  // The tiles of the next 32 landmarks are on their way to registers during this step's products (E: 8 per thread); with the
+  // kernel values of k_nt_g requested ahead of its products: training step of 32 fp32 heads x 784 tokens 313 -> 305 us.
+  const int er = tid >> 2, ei = i0 + er;
+  const float mi = (mu && ei < n) ? mu[(long long)bh * n + ei] : 0.f;
+  float4 ev[2], yv[D / 32];
+  auto fetch = [&](int l0) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int l = l0 + (tid & 3) * 8 + 4 * h;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (ei < n && l < m) {
+        const float* src = E + (long long)ei * lde + l;
+        if (l + 3 < lde && (lde & 3) == 0) v = ld4(src);
+        else {
+          v.x = src[0];
+          if (l + 1 < m) v.y = src[1];
+          if (l + 2 < m) v.z = src[2];
+          if (l + 3 < m) v.w = src[3];
+        }
+      }
+      ev[h] = v;
+    }
+#pragma unroll
+    for (int t = 0; t < D / 32; ++t) {
+      const int idx = tid + t * 256, r = idx / (D / 4), c4 = (idx % (D / 4)) * 4;
+      yv[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (l0 + r < m) yv[t] = ld4(Y + (long long)(l0 + r) * D + c4);
+    }
+  };
+  fetch(0);
   for (int l0 = 0; l0 < m; l0 += 32) {
     __syncthreads();
-    {  // E tile: 64 tokens x 32 landmarks
-      const int r = tid >> 2, cb = (tid & 3) * 8, i = i0 + r;
-      const float mi = (mu && i < n) ? mu[(long long)bh * n + i] : 0.f;
 #pragma unroll
-      for (int k = 0; k < 8; k += 4) {
-        const int l = l0 + cb + k;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i < n && l < m) {
-          if (l + 3 < lde && (lde & 3) == 0) v = ld4(E + (long long)i * lde + l);
-          else {
-            v.x = E[(long long)i * lde + l];
-            if (l + 1 < m) v.y = E[(long long)i * lde + l + 1];
-            if (l + 2 < m) v.z = E[(long long)i * lde + l + 2];
-            if (l + 3 < m) v.w = E[(long long)i * lde + l + 3];
-          }
-          v.x = (l < m) ? v.x - mi : 0.f;
-          v.y = (l + 1 < m) ? v.y - mi : 0.f;
-          v.z = (l + 2 < m) ? v.z - mi : 0.f;
-          v.w = (l + 3 < m) ? v.w - mi : 0.f;
-        }
-        *reinterpret_cast<float4*>(&Es[r][cb + k]) = v;
-      }
+    for (int h = 0; h < 2; ++h) {
+      const int l = l0 + (tid & 3) * 8 + 4 * h;
+      *reinterpret_cast<float4*>(&Es[er][(tid & 3) * 8 + 4 * h]) =
+          make_float4(l < m ? ev[h].x - mi : 0.f, l + 1 < m ? ev[h].y - mi : 0.f, l + 2 < m ? ev[h].z - mi : 0.f, l + 3 < m ? ev[h].w - mi : 0.f);
     }
-    for (int idx = tid; idx < 32 * (D / 4); idx += 256) {
-      const int r = idx / (D / 4), c4 = (idx % (D / 4)) * 4, l = l0 + r;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (l < m) v = ld4(Y + (long long)l * D + c4);
-      *reinterpret_cast<float4*>(&Ys[r][c4]) = v;
+#pragma unroll
+    for (int t = 0; t < D / 32; ++t) {
+      const int idx = tid + t * 256;
+      *reinterpret_cast<float4*>(&Ys[idx / (D / 4)][(idx % (D / 4)) * 4]) = yv[t];
     }
+    if (l0 + 32 < m) fetch(l0 + 32);
     __syncthreads();
 #pragma unroll 2
     for (int ll = 0; ll < 32; ll += 4) {
@@ -932,6 +945,14 @@ __global__ void __launch_bounds__(256) k_nt_g(const TU* __restrict__ U, const fl
   for (int k = 0; k < 4; ++k)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[k][q] = 0.f;
+  float ev[4][4];            // kernel values, on their way during the products
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = i0 + tt * 4 + k, l = l0 + tl + 16 * q;
+      ev[k][q] = (i < n && l < m) ? E[(long long)i * lde + l] : 0.f;
+    }
   for (int c0 = 0; c0 < D; c0 += DK) {
     __syncthreads();
     for (int idx = tid; idx < 64 * (DK / 4); idx += 256) {
@@ -964,7 +985,7 @@ __global__ void __launch_bounds__(256) k_nt_g(const TU* __restrict__ U, const fl
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int l = l0 + tl + 16 * q;
-      if (l < m) G[(long long)i * lde + l] = acc[k][q] * E[(long long)i * lde + l] * inv_lambda;
+      if (l < m) G[(long long)i * lde + l] = acc[k][q] * ev[k][q] * inv_lambda;
       else if (l < lde) G[(long long)i * lde + l] = 0.f;
     }
   }
