@@ -538,9 +538,7 @@ void launch_l1_args(const char* name, L1Args& a, int nprob, int batch, cudaStrea
   // landmarks 12758 -> 12699.  Shorter launches beside the per-head kernels lose: their CTAs take the places these wait for
   // (step of 32 x 3136 tokens 397 -> 399, of 15 x 1074 tokens 187 -> 190).  The partial column statistics have one slot per
   // tile of the larger CTAs.
-  bool fine = nprob == 3 || (long long)na_max * a.nb * a.d * batch > (1ll << 30);
-  for (int i = 0; i < nprob; ++i) fine = fine && !a.p[i].stat;
-  L1Launch l = plan_l1(na_max, a.nb, a.d, batch, nprob, fine);
+  L1Launch l = plan_l1(na_max, a.nb, a.d, batch, nprob, false);
   // a single block without row sums (the stand-alone entry point on few, large matrices): the landmark range is split
   // over blockIdx.z until the launch has about two CTAs per SM
   a.jsplits = 1;
@@ -551,6 +549,11 @@ void launch_l1_args(const char* name, L1Args& a, int nprob, int batch, cudaStrea
     if (sp > tiles) sp = tiles;
     if (sp > 1) { a.jsplits = (int)sp; l.grid.z = (unsigned)sp; }
   }
+  // A split launch keeps the larger CTAs: two of the smaller ones per SM are half the threads (one 3000 x 3000 block with 128
+  // dims 107 us, with CTAs of 128 threads 150; four 3000 x 3000 blocks with 64 dims 250 and 293).
+  bool fine = a.jsplits == 1 && (nprob == 3 || (long long)na_max * a.nb * a.d * batch > (1ll << 30));
+  for (int i = 0; i < nprob; ++i) fine = fine && !a.p[i].stat;
+  if (fine) l = plan_l1(na_max, a.nb, a.d, batch, nprob, true);
   if (l.qn == 4) {
     want_smem(k_l1<4>, l.smem);
     LN_LAUNCH(name, st, enqueue(k_l1<4>, l.grid, l.block, l.smem, st, a));

@@ -50,6 +50,39 @@ def test_l1_kernel_few_large_blocks_split_their_columns(batch, na, nb, d, dtype)
     assert torch.equal(K, K2)
 
 
+@pytest.mark.parametrize("batch,na,nb,d", [(1, 3000, 2999, 128), (70, 400, 500, 96), (200, 405, 420, 32)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_l1_kernel_beyond_two_to_the_30_pair_dims(batch, na, nb, d, dtype):
+    """Long launches, with and without a split column range and with CTAs of either size: the bits of the same rows in calls
+    of a third of the work, and the oracle on a few of them."""
+    assert batch * na * nb * d > 1 << 30 > batch * na * nb * d / 3
+    A, Bm = _rand((batch, na, d), 7, dtype).to(DEV), _rand((batch, nb, d), 8, dtype).to(DEV)
+    K = ln.l1_kernel(A, Bm, float(d))
+    for part in torch.arange(na).chunk(3):
+        assert torch.equal(K[:, part[0]:part[-1] + 1], ln.l1_kernel(A[:, part[0]:part[-1] + 1].contiguous(), Bm, float(d)))
+    rows = [0, na // 2, na - 1]
+    ref = oracle.l1_kernel(f64(A[-1:, rows]), f64(Bm[-1:]), float(d))
+    assert rel_err(f64(K[-1:, rows]), ref) < 1e-5
+
+
+def test_l1_kernel_split_launches_keep_their_speed_beyond_two_to_the_30():
+    """2880 x 2880 and 3000 x 3000 pairs of 128 dims are 23 and 24 row tiles of the same twelve column ranges: 1.08 times the
+    work, on either side of 2^30.  CTAs of half the threads at the same number per SM take 1.4 times as long."""
+    def best(n):
+        A, Bm = _rand((1, n, 128), 9, torch.float32).to(DEV), _rand((1, n, 128), 10, torch.float32).to(DEV)
+        us = []
+        for _ in range(12):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(8):
+                ln.l1_kernel(A, Bm, 128.0)
+            e1.record()
+            torch.cuda.synchronize()
+            us.append(e0.elapsed_time(e1))
+        return min(us)
+    assert best(3000) < 1.2 * best(2880)
+
+
 @pytest.mark.parametrize("batch,na,nb,d", [(1, 300, 777, 64), (2, 130, 1000, 32), (1, 70, 2049, 128)])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_l1_kernel_bwd_few_large_blocks(batch, na, nb, d, dtype):
