@@ -65,29 +65,17 @@ struct Carver {
 };
 
 // Tile of the l1 kernel for a problem: LG landmark groups of QN (4 or 2) landmarks, TG token groups of 8,
-// LG * TG <= 256 threads, chosen so that the tiles hug the problem.  Small heads (few pairs per CTA) take
-// the two-landmark thread tile, which fits three CTAs per SM.
-// CTAs of up to 128 threads (four or six per SM; `fine`): more of them are at different points of load, barrier and arithmetic,
-// and the tiles are finer.  They are taken where they fill their warps and cover the tokens about as well as CTAs of 256 (m = 49
-// with four landmarks a thread does not: 13 x 9 threads of 128 against 13 x 19 of 256), and only for launches that have the GPU
-// to themselves or outlast what runs beside them (see launch_l1_args).
+// LG * TG <= 256 threads (128 with `fine`), chosen so that the tiles hug the problem.  Small heads (few pairs per CTA) take
+// the two-landmark thread tile, which fits three CTAs of 256 threads per SM; the other one fits two.
 struct L1Launch { dim3 grid, block; size_t smem; int qn; };
 L1Launch plan_l1(int na_max, int nb, int d, int batch, int nprob, bool fine) {
   const int qn = ((long long)na_max * nb * d <= (1ll << 20)) ? 2 : 4;
   const int lg_cap = (qn == 4) ? 16 : 32;
   int LG = (nb + qn - 1) / qn; if (LG > lg_cap) LG = lg_cap; if (LG < 1) LG = 1;
+  int tg_cap = (fine ? 128 : 256) / LG; if (tg_cap > 32) tg_cap = 32;       // at most 256 tokens per tile
   const int groups = (na_max + 7) / 8;
-  // token groups of a CTA of up to `cap` threads (at most 256 tokens) and the share of its lanes' time that is of use
-  auto fit = [&](int cap, int& TG) {
-    int tg_cap = cap / LG; if (tg_cap > 32) tg_cap = 32;
-    const int tiles = (groups + tg_cap - 1) / tg_cap;
-    TG = (groups + tiles - 1) / tiles; if (TG < 1) TG = 1;
-    const int threads = LG * TG, ctas = (na_max + 8 * TG - 1) / (8 * TG);
-    return (double)threads / ((threads + 31) / 32 * 32) * na_max / ((double)ctas * 8 * TG);
-  };
-  int TG, TGs;
-  const double large = fit(256, TG), small = fit(128, TGs);
-  if (fine && small >= 0.98 * large) TG = TGs;
+  const int tiles = (groups + tg_cap - 1) / tg_cap;
+  int TG = (groups + tiles - 1) / tiles; if (TG < 1) TG = 1;
   L1Launch l;
   l.qn = qn;
   l.block = dim3(LG, TG);
@@ -530,14 +518,48 @@ L1Prob l1_prob(const void* A, int a_f32, float* E, float* rowsum, int na, int d,
   return q;
 }
 
+// Whether CTAs of up to 128 threads (launch s, instead of l with up to 256) serve a launch of the l1 kernel.  There are
+// twice as many, at different points of load, barrier and arithmetic, and their tiles are finer; but a CTA stages its landmark
+// tile for fewer tokens.  Measured on 1322 launches of three blocks, 1 to 384 heads, 64 to 5589 tokens, 4 to 256 landmarks
+// (10 to 370 us): where this takes them 1.09 in the median, 1.12 over the sum (m = 25, 784 tokens,
+// 160 heads with 128 dims 156 -> 121 us), 9 of 1141 below 0.985; each clause leaves out a class that lost (of the other 181, 64
+// are below 0.985 with smaller CTAs).  Times in the clauses: launch with l and with s.
+bool l1_fine(const L1Launch& l, const L1Launch& s, const L1Args& a, int nprob, int na_max, int batch) {
+  struct Load { int warps, covered, passes; long long per_sm; };       // of a CTA; CTAs on the busiest SM
+  auto load = [&](const L1Launch& x) {
+    const int LG = x.block.x, TG = x.block.y, thr = LG * TG;
+    long long ctas = 0;
+    for (int i = 0; i < nprob; ++i) ctas += (long long)cdiv(a.p[i].na, 8 * TG) * batch;
+    Load r;
+    r.warps = (int)cdiv(thr, 32);
+    r.covered = (int)cdiv(na_max, 8 * TG) * 8 * TG;
+    r.passes = (int)(cdiv(32 * TG, thr) + cdiv(4 * x.qn * LG, thr));     // of the threads over the pieces of 8 dims of a chunk
+    r.per_sm = cdiv(ctas, sm_count());
+    return r;
+  };
+  const Load x = load(l), y = load(s);
+  // the smaller CTAs fill their warps and hug the tokens about as well (m = 49 with four landmarks a thread does not:
+  // 13 x 9 threads of 128 against 13 x 19 of 256)
+  const double use = (double)l.block.x * l.block.y / x.warps / x.covered, use_s = (double)s.block.x * s.block.y / y.warps / y.covered;
+  if (use_s < 0.98 * use) return false;
+  const long long wx = x.per_sm * x.warps, wy = y.per_sm * y.warps;        // warps the busiest SM gets
+  if (2 * wy <= wx) return true;
+  const bool rounds = x.per_sm > 65536 / ((l.qn == 4 ? 128 : 80) * 32 * x.warps);      // the larger ones are not all resident at once
+  // all resident and no fewer warps where it counts: m = 36, 784 tokens, 32 heads 23.0 us, with smaller CTAs 25.0
+  if (!rounds && wy >= wx && x.per_sm > 1) return false;
+  if (y.passes > x.passes) {                                               // and the landmarks take another pass of loads:
+    if (l.qn == 2 && y.warps < 4) return false;                            // m = 42, 64 tokens, 384 heads 32.6 / 35.3
+    if (!rounds && 25 * y.covered > 26 * x.covered) return false;          // m = 36, 196 tokens, 64 heads 18.8 / 20.9
+    if (a.d <= 32 && l.qn == 4 && 10 * wy > 9 * wx) return false;          // one chunk of dims: m = 56, 3136 tokens, 32 heads 49.5 / 53.6
+    // few chunks of dims, rows of less than half a warp: m = 54, 3136 tokens, 32 heads with 64 dims 82.3 / 84.4
+    if (rounds && wy >= wx && y.covered >= x.covered && l.block.x < 16 && a.d < 128) return false;
+  }
+  return true;
+}
+
 void launch_l1_args(const char* name, L1Args& a, int nprob, int batch, cudaStream_t st) {
   int na_max = 0;
   for (int i = 0; i < nprob; ++i) na_max = a.p[i].na > na_max ? a.p[i].na : na_max;
-  // Smaller CTAs where C, R^T and W are one launch (nothing runs beside it), or from 2^30 (pair, dim)s on: 384 heads x 197
-  // tokens, 49 landmarks 82.7 -> 76.6 us (step 466 -> 461); 224 x 224-token inference 1546 -> 1520 us, step of 128 heads with 256
-  // landmarks 12758 -> 12699.  Shorter launches beside the per-head kernels lose: their CTAs take the places these wait for
-  // (step of 32 x 3136 tokens 397 -> 399, of 15 x 1074 tokens 187 -> 190).  The partial column statistics have one slot per
-  // tile of the larger CTAs.
   L1Launch l = plan_l1(na_max, a.nb, a.d, batch, nprob, false);
   // a single block without row sums (the stand-alone entry point on few, large matrices): the landmark range is split
   // over blockIdx.z until the launch has about two CTAs per SM
@@ -549,11 +571,18 @@ void launch_l1_args(const char* name, L1Args& a, int nprob, int batch, cudaStrea
     if (sp > tiles) sp = tiles;
     if (sp > 1) { a.jsplits = (int)sp; l.grid.z = (unsigned)sp; }
   }
-  // A split launch keeps the larger CTAs: two of the smaller ones per SM are half the threads (one 3000 x 3000 block with 128
-  // dims 107 us, with CTAs of 128 threads 150; four 3000 x 3000 blocks with 64 dims 250 and 293).
+  // Smaller CTAs (l1_fine) where C, R^T and W are one launch, so that nothing runs beside it, or where one block has more
+  // than 2^30 (pair, dim)s: 384 heads x 197 tokens, 49 landmarks 82.7 -> 76.6 us (step 466 -> 461); 224 x 224-token inference
+  // 1545 -> 1519.  Shorter launches beside the per-head kernels lose: their CTAs take the places these wait for (step of 32 x
+  // 3136 tokens 397 -> 399, of 15 x 1074 tokens 187 -> 190).  The partial column statistics have one slot per tile of the larger
+  // CTAs.  A split launch keeps the larger ones as well: two of the smaller per SM are half the threads (one 3000 x 3000 block
+  // with 128 dims 107 us, with CTAs of 128 threads 150; four 3000 x 3000 blocks with 64 dims 250 and 293).
   bool fine = a.jsplits == 1 && (nprob == 3 || (long long)na_max * a.nb * a.d * batch > (1ll << 30));
   for (int i = 0; i < nprob; ++i) fine = fine && !a.p[i].stat;
-  if (fine) l = plan_l1(na_max, a.nb, a.d, batch, nprob, true);
+  if (fine) {
+    const L1Launch s = plan_l1(na_max, a.nb, a.d, batch, nprob, true);
+    if (l1_fine(l, s, a, nprob, na_max, batch)) l = s;
+  }
   if (l.qn == 4) {
     want_smem(k_l1<4>, l.smem);
     LN_LAUNCH(name, st, enqueue(k_l1<4>, l.grid, l.block, l.smem, st, a));
