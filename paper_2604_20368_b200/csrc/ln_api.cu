@@ -863,8 +863,8 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
   };
   auto launch_sign_W = [&](cudaStream_t s) {
     // one set: GW is symmetrised, so the row pass carries both roles of L.  Two sets: rows -> pooled queries, columns -> pooled keys
-    LN_LAUNCH("sign_rows_dLW", s, enqueue(k_sign_rows<float, float, float, D>, dim3(cdiv(m, 64), BH), 256, 0, s, LfR, LfC, w.GW, pl.ldm, w.dLW, m, m, 0, nullptr, 1.f));
-    if (two) LN_LAUNCH("sign_cols_dLW", s, enqueue(k_sign_cols<float, float, D>, dim3(1, cdiv(m, 64), BH), 256, 0, s, LfR, LfC, w.GW, pl.ldm, w.dLW2, m, m, (m + 31) / 32 * 32, nullptr, 1.f));
+    LN_LAUNCH("sign_rows_dLW", s, enqueue(k_sign_rows<float, float, float, D>, dim3(cdiv(m, 64), BH), 256, 0, s, LfR, LfC, w.GW, pl.ldm, w.dLW, m, m));
+    if (two) LN_LAUNCH("sign_cols_dLW", s, enqueue(k_sign_cols<float, float, D>, dim3(1, cdiv(m, 64), BH), 256, 0, s, LfR, LfC, w.GW, pl.ldm, w.dLW2, m, m, (m + 31) / 32 * 32));
   };
   // Side stream: the per-head kernel, the landmark-block sign pass and dV (bound by latency and by memory) run beside
   // the sign passes (bound by arithmetic).  The upstream of the key-side block, which the second sign pass waits for,
@@ -923,9 +923,9 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
       else launch2("sign2_dQ_dLC", k_sign2<T, T, 2>, Q, dQ, w.dLCpart);
     }
   } else {
-    if (qrows_f) LN_LAUNCH("sign_rows_dQ", st, enqueue(k_sign_rows<T, float, float, D>, dim3(cdiv(n, 64), BH), 256, 0, st, Q, LfC, w.G, pl.ldm, qrows_f, n, m, 0, nullptr, 1.f));
-    else LN_LAUNCH("sign_rows_dQ", st, enqueue(k_sign_rows<T, float, T, D>, dim3(cdiv(n, 64), BH), 256, 0, st, Q, LfC, w.G, pl.ldm, dQ, n, m, 0, nullptr, 1.f));
-    LN_LAUNCH("sign_cols_dLC", st, enqueue(k_sign_cols<T, float, D>, dim3(ch, cdiv(m, 64), BH), 256, 0, st, Q, LfC, w.G, pl.ldm, w.dLCpart, n, m, pl.rpc, nullptr, 1.f));
+    if (qrows_f) LN_LAUNCH("sign_rows_dQ", st, enqueue(k_sign_rows<T, float, float, D>, dim3(cdiv(n, 64), BH), 256, 0, st, Q, LfC, w.G, pl.ldm, qrows_f, n, m));
+    else LN_LAUNCH("sign_rows_dQ", st, enqueue(k_sign_rows<T, float, T, D>, dim3(cdiv(n, 64), BH), 256, 0, st, Q, LfC, w.G, pl.ldm, dQ, n, m));
+    LN_LAUNCH("sign_cols_dLC", st, enqueue(k_sign_cols<T, float, D>, dim3(ch, cdiv(m, 64), BH), 256, 0, st, Q, LfC, w.G, pl.ldm, w.dLCpart, n, m, pl.rpc));
   }
   if (side.on()) { side.join_mark(st); if (!ntg_on_side && !sign3) launch_ntg_R(st); }
   else { launch_mid(st); launch_sign_W(st); if (!sign3) launch_ntg_R(st); launch_nn_dV(st); }
@@ -946,9 +946,9 @@ int bwd_impl(const ln_problem* p, const Plan& pl, const T* Q, const T* K, const 
       else launch2("sign2_dK_dLR", k_sign2<T, float, 2>, K, w.dKpart, w.dLRpart);
     }
   } else {
-    if (!krows_f) LN_LAUNCH("sign_rows_dK", st, enqueue(k_sign_rows<T, float, T, D>, dim3(cdiv(n, 64), BH), 256, 0, st, K, LfR, w.G2, pl.ldm, dK, n, m, 0, nullptr, 1.f));
-    else LN_LAUNCH("sign_rows_dK", st, enqueue(k_sign_rows<T, float, float, D>, dim3(cdiv(n, 64), BH), 256, 0, st, K, LfR, w.G2, pl.ldm, krows_f, n, m, 0, nullptr, 1.f));
-    LN_LAUNCH("sign_cols_dLR", st, enqueue(k_sign_cols<T, float, D>, dim3(ch, cdiv(m, 64), BH), 256, 0, st, K, LfR, w.G2, pl.ldm, w.dLRpart, n, m, pl.rpc, nullptr, 1.f));
+    if (!krows_f) LN_LAUNCH("sign_rows_dK", st, enqueue(k_sign_rows<T, float, T, D>, dim3(cdiv(n, 64), BH), 256, 0, st, K, LfR, w.G2, pl.ldm, dK, n, m));
+    else LN_LAUNCH("sign_rows_dK", st, enqueue(k_sign_rows<T, float, float, D>, dim3(cdiv(n, 64), BH), 256, 0, st, K, LfR, w.G2, pl.ldm, krows_f, n, m));
+    LN_LAUNCH("sign_cols_dLR", st, enqueue(k_sign_cols<T, float, D>, dim3(ch, cdiv(m, 64), BH), 256, 0, st, K, LfR, w.G2, pl.ldm, w.dLRpart, n, m, pl.rpc));
   }
   // landmark gradient and its way back to the keys
   if (side.on()) side.join(st);      // dV and the landmark-block part are complete

@@ -1020,10 +1020,11 @@ __device__ __forceinline__ bool sign_vec(const float* G, const float* Gk, int ld
 
 // =====================================================================================
 // Sign pass over the landmarks (App. A):  out[i][c] = -sum_l G[i][l] * sign(tok[i][c] - L[l][c])
-// grid (ceil(n/64), BH[, splits]); thread: 4 tokens x D/16 dims, token values held in registers.
-// lper > 0 (a multiple of 32): blockIdx.z takes the landmarks [z lper, (z + 1) lper) and writes the partial sum
-// out[bh][z][n][D] (few, long rows of landmarks: the stand-alone kernel gradient).  Gk != NULL: the factor is formed on
-// the fly as G[i][l] Gk[i][l] gscale (upstream gradient times kernel value over lambda).
+// A CTA per 64 tokens; thread: 4 tokens x D/16 dims, token values held in registers.
+// lper > 0 (a multiple of 32): split z takes the landmarks [z lper, (z + 1) lper) and writes the partial sum
+// out[bh][z][n][D] (few, long rows of landmarks).  Gk != NULL: the factor is formed on the fly as G[i][l] Gk[i][l] gscale
+// (upstream gradient times kernel value over lambda).  k_sign_rows and k_sign_cols pass NULL, which folds the tests away.
+// k_sign_both, where Gk is never NULL, keeps them: without, its loads are scheduled another way (two 1024 x 1024 blocks 36.5 -> 37.4 us).
 template <typename TT, typename TL, typename TO, int D>
 __device__ __forceinline__ void sign_rows_tile(float* smem, int tile, int bh, int split, int nsplits, const TT* __restrict__ tok,
                                                const TL* __restrict__ Lm, const float* __restrict__ G, int ldg, TO* __restrict__ out,
@@ -1118,14 +1119,17 @@ __device__ __forceinline__ void sign_rows_tile(float* smem, int tile, int bh, in
   }
 }
 template <int D> constexpr int kSignSmem = 32 * (D + 4) + 64 * 36;      // floats, the larger of the two passes
+// The tile on its way takes 13 to 24 registers, which left one CTA per SM instead of two at 128 dims (158 registers; two sets of
+// 64 landmarks on 128 heads x 1600 tokens, fp32: pass over the landmarks 240 us without the tile, 259 with it).  Bounded to the
+// CTAs per SM that measured best: 211 us, over the tokens 271 without, 248 with, 223 bounded; at 64 dims and 128 landmarks
+// 238 / 214 / 207 and 235 / 229 / 225; 256 heads x 784 tokens, 32 dims 152 / 138 / 130 and 147 / 132 / 130.
 template <typename TT, typename TL, typename TO, int D>
-__global__ void __launch_bounds__(256) k_sign_rows(const TT* __restrict__ tok, const TL* __restrict__ Lm,
-                                                   const float* __restrict__ G, int ldg, TO* __restrict__ out,
-                                                   int n, int m, int lper = 0, const float* __restrict__ Gk = nullptr,
-                                                   float gscale = 1.f) {
+__global__ void __launch_bounds__(256, D == 32 ? 3 : 2) k_sign_rows(const TT* __restrict__ tok, const TL* __restrict__ Lm,
+                                                                     const float* __restrict__ G, int ldg, TO* __restrict__ out,
+                                                                     int n, int m) {
   pdl_wait();
   __shared__ __align__(16) float smem[kSignSmem<D>];
-  sign_rows_tile<TT, TL, TO, D>(smem, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z, tok, Lm, G, ldg, out, n, m, lper, Gk, gscale);
+  sign_rows_tile<TT, TL, TO, D>(smem, blockIdx.x, blockIdx.y, 0, 1, tok, Lm, G, ldg, out, n, m, 0, nullptr, 1.f);
 }
 
 // =====================================================================================
@@ -1217,13 +1221,12 @@ __device__ __forceinline__ void sign_cols_tile(float* smem, int chunk, int nchun
   }
 }
 template <typename TT, typename TL, int D>
-__global__ void __launch_bounds__(256) k_sign_cols(const TT* __restrict__ tok, const TL* __restrict__ Lm,
-                                                   const float* __restrict__ G, int ldg, float* __restrict__ part,
-                                                   int n, int m, int rpc, const float* __restrict__ Gk = nullptr,
-                                                   float gscale = 1.f) {
+__global__ void __launch_bounds__(256, D == 128 ? 2 : 3) k_sign_cols(const TT* __restrict__ tok, const TL* __restrict__ Lm,
+                                                                     const float* __restrict__ G, int ldg, float* __restrict__ part,
+                                                                     int n, int m, int rpc) {
   pdl_wait();
   __shared__ __align__(16) float smem[kSignSmem<D>];
-  sign_cols_tile<TT, TL, D>(smem, blockIdx.x, gridDim.x, blockIdx.y, blockIdx.z, tok, Lm, G, ldg, part, n, m, rpc, Gk, gscale);
+  sign_cols_tile<TT, TL, D>(smem, blockIdx.x, gridDim.x, blockIdx.y, blockIdx.z, tok, Lm, G, ldg, part, n, m, rpc, nullptr, 1.f);
 }
 
 // Both passes of the stand-alone kernel gradient in one launch: neither fills the GPU's places for long on a few matrices,
