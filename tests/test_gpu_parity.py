@@ -50,16 +50,20 @@ def test_l1_kernel_few_large_blocks_split_their_columns(batch, na, nb, d, dtype)
     assert torch.equal(K, K2)
 
 
-@pytest.mark.parametrize("batch,na,nb,d", [(1, 3000, 2999, 128), (70, 400, 500, 96), (200, 405, 420, 32)])
+@pytest.mark.parametrize("batch,na,nb,d", [(1, 3000, 2999, 128), (80, 400, 500, 96), (200, 405, 420, 32)])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 def test_l1_kernel_beyond_two_to_the_30_pair_dims(batch, na, nb, d, dtype):
-    """Long launches, with and without a split column range and with CTAs of either size: the bits of the same rows in calls
-    of a third of the work, and the oracle on a few of them."""
+    """Long launches, with a split column range (CTAs of 256 threads) and without (128): the bits of the same rows, and of
+    their sums, in calls of a third of the work, and the oracle on a few of them."""
     assert batch * na * nb * d > 1 << 30 > batch * na * nb * d / 3
     A, Bm = _rand((batch, na, d), 7, dtype).to(DEV), _rand((batch, nb, d), 8, dtype).to(DEV)
     K = ln.l1_kernel(A, Bm, float(d))
+    K2, rs = ln.l1_kernel(A, Bm, float(d), want_rowsum=True)
+    assert torch.equal(K, K2)
     for part in torch.arange(na).chunk(3):
-        assert torch.equal(K[:, part[0]:part[-1] + 1], ln.l1_kernel(A[:, part[0]:part[-1] + 1].contiguous(), Bm, float(d)))
+        i, j = int(part[0]), int(part[-1]) + 1
+        Kp, rsp = ln.l1_kernel(A[:, i:j].contiguous(), Bm, float(d), want_rowsum=True)
+        assert torch.equal(K[:, i:j], Kp) and torch.equal(rs[:, i:j], rsp)
     rows = [0, na // 2, na - 1]
     ref = oracle.l1_kernel(f64(A[-1:, rows]), f64(Bm[-1:]), float(d))
     assert rel_err(f64(K[-1:, rows]), ref) < 1e-5
@@ -108,10 +112,13 @@ def test_l1_kernel_exact_properties():
     assert torch.equal(torch.diagonal(K, dim1=1, dim2=2), torch.ones(2, 90, device=DEV))
 
 
-@pytest.mark.parametrize("batch,na,nb,d", [(2, 197, 49, 64), (1, 70, 130, 32), (1, 33, 5, 128), (3, 1, 1, 32)])
+@pytest.mark.parametrize("batch,na,nb,d", [(2, 197, 49, 64), (1, 70, 130, 32), (1, 33, 5, 128), (3, 1, 1, 32),
+                                           (60, 320, 197, 32), (60, 320, 196, 64), (2, 130, 132, 64), (1, 70, 260, 128)])
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("recompute", [False, True])
 def test_l1_kernel_bwd(batch, na, nb, d, dtype, recompute):
+    """Rows split over the columns (few row tiles) and written directly (300 row tiles, with several token chunks and column
+    tiles beside them); rows of dK read in quads (nb a multiple of four) and one by one."""
     A, Bm = _rand((batch, na, d), 4, dtype), _rand((batch, nb, d), 5, dtype)
     if na > 4 and nb > 2:                 # exact ties: sign(0) = 0 on both sides
         A[0, 3] = Bm[0, 1]
@@ -406,9 +413,19 @@ def test_fp32_storage_token_chunks(gh, gw, prefix, d, B):
 @pytest.mark.parametrize("gh,gw,prefix,d,dtype,B", [(8, 8, 1, 64, "f32", 1), (9, 14, 0, 32, "f32", 2), (14, 14, 1, 64, "bf16", 56),
                                                     (9, 8, 0, 128, "bf16", 56)])
 def test_kernel_blocks_in_one_launch(mh, mw, gh, gw, prefix, d, dtype, B):
-    """C, R^T and W from one launch (fp32 storage, or more than 220 bf16 heads of few tokens), whose CTAs have up to 128 threads
-    where these fill their warps: one to 49 landmark groups, token tiles with and without a remainder."""
+    """C, R^T and W from one launch (fp32 storage, or more than 220 bf16 heads of few tokens) with two landmarks a thread, in CTAs of
+    up to 128 threads or 256: one to 32 landmark groups, token tiles with and without a remainder."""
     cfg = synth.Config("one_launch", B=B, H=4, d=d, m=mh * mw, T=3, gh=gh, gw=gw, mh=mh, mw=mw, prefix=prefix, dtype=dtype, seed=5 + mh * mw)
+    _run_case(cfg, heads=[0, 4 * B - 1], intermediates=True)
+
+
+@pytest.mark.parametrize("mh,mw,gh,gw,prefix,d,B", [(4, 8, 28, 28, 0, 64, 1), (6, 9, 28, 28, 0, 64, 8), (8, 8, 20, 20, 1, 64, 16),
+                                                    (5, 5, 28, 28, 0, 128, 40), (8, 16, 41, 39, 0, 128, 2),
+                                                    (6, 6, 28, 28, 0, 64, 8), (7, 8, 56, 56, 0, 32, 8), (6, 9, 56, 56, 0, 64, 8)])
+def test_kernel_blocks_with_four_landmarks_a_thread(mh, mw, gh, gw, prefix, d, B):
+    """The same from 2^20 (pair, dim)s per head on: five shapes that take CTAs of up to 128 threads (few heads, one and several rounds
+    of CTAs, as many and more passes of loads) and three that keep 256."""
+    cfg = synth.Config("four_a_thread", B=B, H=4, d=d, m=mh * mw, T=2, gh=gh, gw=gw, mh=mh, mw=mw, prefix=prefix, dtype="f32", seed=9 + mh * mw)
     _run_case(cfg, heads=[0, 4 * B - 1], intermediates=True)
 
 
