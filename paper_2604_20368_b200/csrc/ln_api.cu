@@ -125,9 +125,13 @@ bool make_plan(const ln_problem* p, Plan* pl) {
   int rpc = (p->n + want - 1) / want;
   if (rpc < 256) rpc = 256;
   // fp32 storage: where chunks of 256 tokens are fewer than two CTAs per SM the product is a chain of eight 32-token steps on
-  // a part of the chip; shorter chunks then, down to 64 tokens and for up to three CTAs per SM (three heads x 196 tokens
-  // 3 -> 12 CTAs, 32 heads x 784 tokens 128 -> 416; figures at k_tn).  bf16 storage keeps its chunks: its ring of three
-  // stages hides the loads, and the order of its sums stays as it was.
+  // a part of the chip; shorter chunks then, down to 64 tokens and for three CTAs per SM or somewhat more (three heads x 196
+  // tokens 3 -> 12 CTAs, 32 heads x 784 tokens 128 -> 416; figures at k_tn).  The same chunks serve the sign pass over the
+  // tokens at 32 dims and with two landmark sets (six heads x 3136 tokens, 32 dims 25 -> 19 us; two sets on two heads x 2025
+  // tokens, 128 dims 54 -> 17).  Those who add the partial results up have more of them (k_mid_fwd + k_mid_bwd of 32 heads x
+  // 784 tokens 137 -> 144 us, k_reduce3 of 64 heads with 32 dims 8.5 -> 10.4), less than the passes gain: steps and inference
+  // of 1 to 221 heads with up to 256 landmarks run at 1.01 to 1.33 times the speed, the tiles on their way included.  bf16
+  // storage keeps its chunks: its ring of three stages hides the loads, and the order of its sums stays as it was.
   if (p->dtype == LN_F32 && (long long)pl->BH * mblk * ((p->n + rpc - 1) / rpc) < 2ll * kSMs) {
     int parts = (3 * kSMs + pl->BH * mblk - 1) / (pl->BH * mblk);
     if (parts > 32) parts = 32;
@@ -521,9 +525,9 @@ L1Prob l1_prob(const void* A, int a_f32, float* E, float* rowsum, int na, int d,
 // Whether CTAs of up to 128 threads (launch s, instead of l with up to 256) serve a launch of the l1 kernel.  There are
 // twice as many, at different points of load, barrier and arithmetic, and their tiles are finer; but a CTA stages its landmark
 // tile for fewer tokens.  Measured on 1322 launches of three blocks, 1 to 384 heads, 64 to 5589 tokens, 4 to 256 landmarks
-// (10 to 370 us): where this takes them 1.09 in the median, 1.12 over the sum (m = 25, 784 tokens,
-// 160 heads with 128 dims 156 -> 121 us), 9 of 1141 below 0.985; each clause leaves out a class that lost (of the other 181, 64
-// are below 0.985 with smaller CTAs).  Times in the clauses: launch with l and with s.
+// (10 to 370 us): where this takes them 1.09 in the median, 1.12 over the sum (m = 25, 784 tokens, 160 heads with 128 dims
+// 156 -> 121 us), 9 of 1141 below 0.985; each clause leaves out a class that lost (of the other 181, 64 are below 0.985 with
+// smaller CTAs).  Times in the clauses: launch with l and with s.
 bool l1_fine(const L1Launch& l, const L1Launch& s, const L1Args& a, int nprob, int na_max, int batch) {
   struct Load { int warps, covered, passes; long long per_sm; };       // of a CTA; CTAs on the busiest SM
   auto load = [&](const L1Launch& x) {
@@ -572,11 +576,13 @@ void launch_l1_args(const char* name, L1Args& a, int nprob, int batch, cudaStrea
     if (sp > 1) { a.jsplits = (int)sp; l.grid.z = (unsigned)sp; }
   }
   // Smaller CTAs (l1_fine) where C, R^T and W are one launch, so that nothing runs beside it, or where one block has more
-  // than 2^30 (pair, dim)s: 384 heads x 197 tokens, 49 landmarks 82.7 -> 76.6 us (step 466 -> 461); 224 x 224-token inference
-  // 1545 -> 1519.  Shorter launches beside the per-head kernels lose: their CTAs take the places these wait for (step of 32 x
-  // 3136 tokens 397 -> 399, of 15 x 1074 tokens 187 -> 190).  The partial column statistics have one slot per tile of the larger
-  // CTAs.  A split launch keeps the larger ones as well: two of the smaller per SM are half the threads (one 3000 x 3000 block
-  // with 128 dims 107 us, with CTAs of 128 threads 150; four 3000 x 3000 blocks with 64 dims 250 and 293).
+  // than 2^30 (pair, dim)s (C and R^T in one launch: each of them): 384 heads x 197 tokens, 49 landmarks 82.7 -> 76.6 us (step
+  // 469 -> 463); 224 x 224-token inference 1548 -> 1522.  Shorter launches beside the per-head kernels lose: their CTAs take the
+  // places these wait for (step of 32 x 3136 tokens 397 -> 399, of 15 x 1074 tokens 187 -> 190).  Just above 2^30, with more than
+  // 64 landmarks and 128 dims, some still do (230 sizes in up to seven rounds of CTAs: median 1.016, a tenth below 0.995, five
+  // heads x 18270 tokens 0.95), and nothing in the sizes tells them apart.  The partial column statistics have one slot per
+  // tile of the larger CTAs.  A split launch keeps the larger ones as well: two of the smaller per SM are half the threads (one
+  // 3000 x 3000 block with 128 dims 107 us, with CTAs of 128 threads 150; four 3000 x 3000 blocks with 64 dims 250 and 293).
   bool fine = a.jsplits == 1 && (nprob == 3 || (long long)na_max * a.nb * a.d * batch > (1ll << 30));
   for (int i = 0; i < nprob; ++i) fine = fine && !a.p[i].stat;
   if (fine) {

@@ -65,8 +65,8 @@ __device__ __forceinline__ void l1_fetch8(const void* base, bool f32, long long 
   }
 }
 
-// QN = landmarks per thread: 4 (128 registers, two CTAs per SM) for large problems; 2 (three CTAs per
-// SM) where a CTA lives too briefly for two of them to hide each other's loads and epilogues.
+// QN = landmarks per thread: 4 (128 registers, two CTAs of 256 threads per SM or four of 128) for large problems; 2 (three or
+// six) where a CTA lives too briefly for two of them to hide each other's loads and epilogues.
 template <int QN>
 __global__ void __launch_bounds__(256, QN == 4 ? 2 : 3) k_l1(const L1Args args) {
   pdl_wait();
